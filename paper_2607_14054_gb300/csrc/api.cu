@@ -32,10 +32,15 @@ struct Tune {
     int N, W, algo, flags;
 };
 
+// The library's defaults: N = 64, W = 4 (tiles of 8,192 samples); N given alone
+// takes W = 8.
 bool resolve_tuning(const sos_tuning* t, Tune* out) {
-    Tune r{32, 8, 1, 0};
+    Tune r{64, 4, 1, 0};
     if (t) {
-        if (t->n_blocks) r.N = t->n_blocks;
+        if (t->n_blocks) {
+            r.N = t->n_blocks;
+            r.W = 8;
+        }
         if (t->warps) r.W = t->warps;
         if (t->algo) r.algo = t->algo;
         r.flags = t->flags;
@@ -44,6 +49,19 @@ bool resolve_tuning(const sos_tuning* t, Tune* out) {
     if (!forward_supported(r.N, r.W) || !pipe_supported(r.N)) return false;
     *out = r;
     return true;
+}
+
+// The backward's: N = 32, W = 8 (the same tiles) where the call leaves N to
+// the library.  Its shared memory per warp, K + 2 groups, allows twice the
+// warps of N = 64.
+sos_tuning backward_tuning(const sos_tuning* t) {
+    sos_tuning r{0, 0, 0, 0};
+    if (t) r = *t;
+    if (r.n_blocks == 0) {
+        r.n_blocks = 32;
+        if (r.warps == 0) r.warps = 8;
+    }
+    return r;
 }
 
 // SMs of the current device (cached per device); 0 if unknown.
@@ -59,12 +77,11 @@ int device_sms() {
 
 constexpr int kPipeCtasPerSm = 2;
 
-// Segment length: long enough that the warm-up before each segment is a small
-// fraction of it, short enough that the segments of the whole call keep every
+// Tile length: long enough that the warm-up before each tile is a small
+// fraction of it, short enough that the tiles of the whole call keep every
 // consumer busy: each pipeline CTA (between 8 and 64 groups of 32 N), or, for
-// the warp-segment kernel, each resident warp (at least 8192 samples, so that
-// horizons up to 4096 samples qualify as with the pipeline, and at most 64
-// groups).
+// the warp-segment kernel, each resident warp (at least 8192 samples and at
+// most 64 groups; it cuts its own segments, Params::wseg).
 // CTAs per SM of a warp-segment launch: the tuning's request (flag bits
 // 8..11), at most as many as fit; 0 = as many as fit.
 int warpseg_ctas(int N, int algo, int flags) {
@@ -182,6 +199,16 @@ sos_status setup(int32_t n_channels, int32_t kmax, const int64_t* lengths_host, 
     p->algo = tu.algo;
     p->seg = segment_length(total_len, tu.N, tu.algo, tu.flags,
                             (tu.flags & SOS_FLAG_SECTION_PIPELINE) == 0);
+    {
+        const int64_t group = 32LL * tu.N;
+        const int64_t sms = device_sms() > 0 ? device_sms() : 148;
+        const int occ = warpseg_ctas(tu.N, tu.algo, tu.flags);
+        const int64_t warps = sms * (occ > 0 ? occ : 1) * warpseg_warps_per_cta();
+        p->fair = (total_len + warps - 1) / warps;
+        int64_t g = (p->fair + group - 1) / group;
+        g = g < 1 ? 1 : g > 64 ? 64 : g;
+        p->wseg = g * group;
+    }
     p->total = total_len;
     *tiles_out = tiles;
     *total_len_out = total_len;
@@ -606,6 +633,8 @@ extern "C" {
 
 size_t sos_backward_workspace_size(int32_t n_channels, int32_t kmax, const int64_t* lengths_host,
                                    const sos_tuning* tuning) {
+    const sos_tuning bt = backward_tuning(tuning);
+    tuning = &bt;
     const size_t base = sos_workspace_size(n_channels, kmax, lengths_host, tuning);
     if (base == 0) return 0;
     Tune tu;
@@ -621,6 +650,8 @@ sos_status sos_filter_backward(const float* x, const double* sos, const int32_t*
                                const float* grad_zf, float* grad_x, double* grad_sos,
                                float* grad_zi, void* workspace, size_t ws_bytes,
                                const sos_tuning* tuning, void* stream) {
+    const sos_tuning bt = backward_tuning(tuning);
+    tuning = &bt;
     Params p{};
     int64_t tiles = 0, total = 0;
     sos_status st = setup(n_channels, kmax, lengths_host, workspace, ws_bytes, tuning, &p, &tiles,

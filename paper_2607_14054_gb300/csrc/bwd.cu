@@ -38,7 +38,7 @@
 // Groups are anchored at the segment's top (the channel's end, or the end of
 // the adjoint warm-up), so dL/dzf enters at a group boundary.  The channel's
 // first group may then start before sample 0: its inputs there are zero and
-// zi enters at the group-relative position of sample 0 (pipe_section's INJ).
+// zi enters at the group-relative position of sample 0 (lane_section's INJ).
 #include "pipe_section.cuh"
 #include "sos_pipe.cuh"
 
@@ -169,11 +169,9 @@ __device__ __forceinline__ void bw_forward_group(const Params& p, const SegGeom&
                 zi1 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 0] * gi;
                 zi2 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 1] * gi;
             }
-            pipe_section<N, FACT, false, true>(v, ab, b0, cf->phi_pow, lp, z.x, z.y, false, 0,
-                                               nullptr, nullptr, 1.f, pinj, zi1, zi2);
+            lane_section<N, FACT, true>(v, ab, b0, cf->phi_pow, lp, z.x, z.y, pinj, zi1, zi2);
         } else {
-            pipe_section<N, FACT, false>(v, ab, b0, cf->phi_pow, lp, z.x, z.y, false, 0, nullptr,
-                                         nullptr, 1.f);
+            lane_section<N, FACT, false>(v, ab, b0, cf->phi_pow, lp, z.x, z.y);
         }
         __syncwarp();
         if (lane == 0) zs[k] = z;

@@ -37,14 +37,15 @@ template <int N, bool FACT, bool CR, bool ZFK>
 __device__ __forceinline__ void pipe_segment_section(const Params& p, const SegGeom& sg, int k,
                                                      PipeShared& sh, float* ring, int& s,
                                                      unsigned& use, const float4 ab,
-                                                     const float4 misc, const float4 lp) {
+                                                     const float4 misc) {
     using SL = SlotLayout<N>;
     const int lane = threadIdx.x & 31;
     const float4* phi = sh.phi[k];
+    const float2 cpl = make_float2(sh.phi[k][7].x, sh.phi[k][7].y);
     // the state entering the segment: zi (scaled by 1/G_k when b0 is
     // factored) for the channel's first segment, zero state otherwise
     float Z1 = 0.f, Z2 = 0.f;
-    if (sg.si == 0 && p.zi) {
+    if (sg.cstart == 0 && p.zi) {
         const float gi = FACT ? misc.z : 1.f;
         Z1 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 0] * gi;
         Z2 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 1] * gi;
@@ -68,29 +69,24 @@ __device__ __forceinline__ void pipe_segment_section(const Params& p, const SegG
         pipe_wait(p, &sh.bar[s][k], use & 1u, lane, sh.limit);
         float* row = ring + s * SL::kFloats + lane * SL::kRow;
         const bool zf_owner = ZG && lane == owner;
-        float v[N];
-#pragma unroll
-        for (int q = 0; q < N / 4; ++q) {
-            const float4 t = *reinterpret_cast<const float4*>(row + 4 * q);
-            v[4 * q + 0] = t.x;
-            v[4 * q + 1] = t.y;
-            v[4 * q + 2] = t.z;
-            v[4 * q + 3] = t.w;
-        }
-        if (!CR)
-            pipe_section<N, FACT, ZG>(v, ab, misc.x, phi, lp, Z1, Z2, zf_owner, mq, row, zf_dst,
-                                      (ZG && FACT) ? G : 1.f);
-        else
+        const float Gz = (ZG && FACT) ? G : 1.f;
+        if constexpr (!CR) {
+            QChunk<N> v;
+            row_to_q<N>(v, row);
+            pipe_section<N, FACT, ZG>(v, ab, misc.x, phi, cpl, Z1, Z2, zf_owner, mq, row, zf_dst, Gz);
+            if (FACT && last_k) q_to_row<N, true>(v, row, G);
+            else q_to_row<N, false>(v, row);
+        } else {
+            float v[N];
+            row_to_chunk<N>(v, row);
             pipe_section_cr<N, FACT, ZG>(v, ab, misc.x, sh.cr[k], Z1, Z2, zf_owner, mq, row,
-                                         zf_dst, (ZG && FACT) ? G : 1.f);
-        if (FACT && last_k) {
+                                         zf_dst, Gz);
+            if (FACT && last_k) {
 #pragma unroll
-            for (int m = 0; m < N; ++m) v[m] *= G;
+                for (int m = 0; m < N; ++m) v[m] *= G;
+            }
+            chunk_to_row<N>(v, row);
         }
-#pragma unroll
-        for (int q = 0; q < N / 4; ++q)
-            *reinterpret_cast<float4*>(row + 4 * q) =
-                make_float4(v[4 * q + 0], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
         __syncwarp();
         pipe_arrive(&sh.bar[s][k + 1]);
         if (++s == kPipeRing) {
@@ -209,7 +205,7 @@ __global__ void __launch_bounds__(2 * kPipeThreads, 1) sos_pipe_kernel(Params p)
         // ---- section k = warp - 1 ----
         const int k = warp - 1;
         int cur_c = -1;
-        float4 ab = make_float4(0.f, 0.f, 0.f, 0.f), misc = ab, lp = ab;
+        float4 ab = make_float4(0.f, 0.f, 0.f, 0.f), misc = ab;
         for (int64_t d = d0; d < total; d += dstep) {
             const SegGeom sg = seg_geom<PC::kGroup>(p, d);
             if (k < sg.K) {
@@ -217,9 +213,8 @@ __global__ void __launch_bounds__(2 * kPipeThreads, 1) sos_pipe_kernel(Params p)
                     const Coef32* cf = p.c32 + (int64_t)sg.c * p.kmax + k;
                     ab = __ldg(&cf->ab);
                     misc = __ldg(&cf->misc);
-                    lp = __ldg(&cf->lane_pow[lane]);
                     __syncwarp();
-                    if (lane < 5) sh.phi[k][lane] = __ldg(&cf->phi_pow[lane]);
+                    if (lane < 8) sh.phi[k][lane] = __ldg(&cf->phi_c[0] + lane);
                     if (lane < 14) sh.cr[k][lane] = __ldg(&cf->cr_lv[0] + lane);
                     __syncwarp();
                     cur_c = sg.c;
@@ -228,16 +223,16 @@ __global__ void __launch_bounds__(2 * kPipeThreads, 1) sos_pipe_kernel(Params p)
                 const bool fact = p.chan[sg.c].mode != 0;
                 if (fact && cr)
                     pipe_segment_section<N, true, true, ZFK>(p, sg, k, sh, ring, s, use, ab,
-                                                             misc, lp);
+                                                             misc);
                 else if (fact)
                     pipe_segment_section<N, true, false, ZFK>(p, sg, k, sh, ring, s, use, ab,
-                                                             misc, lp);
+                                                             misc);
                 else if (cr)
                     pipe_segment_section<N, false, true, ZFK>(p, sg, k, sh, ring, s, use, ab,
-                                                             misc, lp);
+                                                             misc);
                 else
                     pipe_segment_section<N, false, false, ZFK>(p, sg, k, sh, ring, s, use, ab,
-                                                             misc, lp);
+                                                             misc);
             } else {
                 // past the channel's K: pass the groups through
                 for (int g = 0; g < sg.ngroups; ++g) {

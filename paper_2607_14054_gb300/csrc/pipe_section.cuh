@@ -5,6 +5,7 @@
 // by the forward section pipeline and, on time-reversed data, by the adjoint.
 #pragma once
 
+#include "sos_f2.cuh"
 #include "sos_pipe.cuh"
 
 namespace sosf {
@@ -44,51 +45,267 @@ __device__ __forceinline__ void row_to_chunk(float (&v)[N], const float* row) {
 }
 
 
-// One section over one group, lane chunk v[] in registers, from the group's
-// incoming DF2T state (Z1, Z2) (scaled by 1/G_k when b0 is factored); leaves
-// the group's outgoing state in (Z1, Z2).  ZF: the group holds the channel's
-// last sample (at element mq of the chunk of the lane where zf_owner is set),
-// whose DF2T state goes to zf_dst; a separate instantiation, so that other
-// groups do not run the selects it needs.  s_own: the lane's row (N floats,
-// 16-byte aligned), scratch for DFS.
-// INJ: a DF2T state (zi1, zi2) enters at group-relative sample pinj instead
-// of the group start (the inputs before it being zero): added to the
-// all-pole input at pinj and pinj + 1 (the backward's recompute of a
-// channel's first group, whose grid is anchored elsewhere).
-// DFS: extended precision for ill-conditioned sections: the lane scan and the
-// fold run in double-float, with the powers' low parts phi_lo and lpl beside
-// phi and lp, and the in-lane recursions add the low parts alo of a1, a2
-// (the samples stay FP32).
-// AL: the in-lane recursions add the low parts alo of a1, a2 (a section
-// whose poles FP32 coefficients would displace noticeably; implied by DFS).
-template <int N, bool FACT, bool ZF = false, bool INJ = false, bool DFS = false, bool AL = DFS>
-__device__ __forceinline__ void pipe_section(float (&v)[N], const float4 ab, const float b0,
-                                             const float4* phi, const float4 lp, float& Z1,
-                                             float& Z2, bool zf_owner, int mq, float* s_own,
-                                             float* zf_dst, float G, int pinj = -1,
-                                             float zi1 = 0.f, float zi2 = 0.f,
-                                             const float4* phi_lo = nullptr,
-                                             float4 lpl = {0.f, 0.f, 0.f, 0.f},
-                                             float2 alo = {0.f, 0.f}) {
+// A lane's chunk of N samples as packed pairs of quarter chunks (Q = N/4):
+// u[m] = (v[m], v[m + Q]), w[m] = (v[m + 2Q], v[m + 3Q]).
+template <int N>
+struct QChunk {
+    f2x u[N / 4], w[N / 4];
+};
+
+template <int N>
+__device__ __forceinline__ void row_to_q(QChunk<N>& v, const float* row) {
+    constexpr int Q = N / 4;
+#pragma unroll
+    for (int q = 0; q < Q; q += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(row + q);
+        const float4 b = *reinterpret_cast<const float4*>(row + Q + q);
+        const float4 c = *reinterpret_cast<const float4*>(row + 2 * Q + q);
+        const float4 d = *reinterpret_cast<const float4*>(row + 3 * Q + q);
+        v.u[q + 0] = f2_pack(a.x, b.x);
+        v.u[q + 1] = f2_pack(a.y, b.y);
+        v.u[q + 2] = f2_pack(a.z, b.z);
+        v.u[q + 3] = f2_pack(a.w, b.w);
+        v.w[q + 0] = f2_pack(c.x, d.x);
+        v.w[q + 1] = f2_pack(c.y, d.y);
+        v.w[q + 2] = f2_pack(c.z, d.z);
+        v.w[q + 3] = f2_pack(c.w, d.w);
+    }
+}
+
+// The chunk to the lane's row, every sample times `scale` (SC).
+template <int N, bool SC>
+__device__ __forceinline__ void q_to_row(const QChunk<N>& v, float* row, float scale = 1.f) {
+    constexpr int Q = N / 4;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const f2x* t = h ? v.w : v.u;
+#pragma unroll
+        for (int q = 0; q < Q; q += 4) {
+            float4 a, b;
+            f2_unpack(t[q + 0], a.x, b.x);
+            f2_unpack(t[q + 1], a.y, b.y);
+            f2_unpack(t[q + 2], a.z, b.z);
+            f2_unpack(t[q + 3], a.w, b.w);
+            if (SC) {
+                a = make_float4(a.x * scale, a.y * scale, a.z * scale, a.w * scale);
+                b = make_float4(b.x * scale, b.y * scale, b.z * scale, b.w * scale);
+            }
+            *reinterpret_cast<float4*>(row + 2 * Q * h + q) = a;
+            *reinterpret_cast<float4*>(row + 2 * Q * h + Q + q) = b;
+        }
+    }
+}
+
+// v[mq] and v[mq - 1] (0 when mq = 0) for a run-time mq, through the lane's
+// row as scratch (N floats, 16-byte aligned).
+template <int N>
+__device__ __forceinline__ void pick_q(const QChunk<N>& v, int mq, float* row, float& q0,
+                                       float& q1) {
+    q_to_row<N, false>(v, row);
+    q0 = row[mq];
+    q1 = mq >= 1 ? row[mq - 1] : 0.f;
+}
+
+// The DF2T states entering a lane's quarters (zu: quarters 0 and 1, zw: 2 and
+// 3) from the quarters' zero-state outgoing states (e*u, e*w) and, with ST,
+// the group's incoming state (Z1, Z2) (zero otherwise): the quarters joined
+// into halves and lanes, the lanes scanned (S4 (ii), z_{l+1} = Phi z_l + s_l),
+// the lane's incoming state passed on from quarter to quarter, all in the
+// basis s1 = z1, s2 = (z2 - t z1) / w (t = a1/2, cpl = (w, 1/w)) that phi is
+// given in.  Lane 0 starts the scan from the group's state, which so reaches
+// every lane without a table of Phi^lane.
+template <bool ST>
+__device__ __forceinline__ void join_states(f2x e1u, f2x e2u, f2x e1w, f2x e2w, float Z1, float Z2,
+                                            float t, const float2 cpl, const float4* phi, f2x& zu1,
+                                            f2x& zu2, f2x& zw1, f2x& zw2) {
     const int lane = threadIdx.x & 31;
-    const float a1 = ab.x, a2 = ab.y, b1 = ab.z, b2 = ab.w;
+    const f2x nt = f2_dup(-t), iw = f2_dup(cpl.y);
+    e2u = f2_mul(f2_fma(nt, e1u, e2u), iw);
+    e2w = f2_mul(f2_fma(nt, e1w, e2w), iw);
+    float s01, s11, s02, s12, s21, s31, s22, s32;
+    f2_unpack(e1u, s01, s11);
+    f2_unpack(e2u, s02, s12);
+    f2_unpack(e1w, s21, s31);
+    f2_unpack(e2w, s22, s32);
+    const float4 hp = phi[5], qp = phi[6];
+    const float A1 = fmaf(qp.x, s01, fmaf(qp.y, s02, s11));
+    const float A2 = fmaf(qp.z, s01, fmaf(qp.w, s02, s12));
+    const float B1 = fmaf(qp.x, s21, fmaf(qp.y, s22, s31));
+    const float B2 = fmaf(qp.z, s21, fmaf(qp.w, s22, s32));
+    float S1 = fmaf(hp.x, A1, fmaf(hp.y, A2, B1));
+    float S2 = fmaf(hp.z, A1, fmaf(hp.w, A2, B2));
+    const float C2 = ST ? fmaf(-t, Z1, Z2) * cpl.y : 0.f;
+    if (ST && lane == 0) {
+        const float4 h = phi[0];
+        S1 = fmaf(h.x, Z1, fmaf(h.y, C2, S1));
+        S2 = fmaf(h.z, Z1, fmaf(h.w, C2, S2));
+    }
+#pragma unroll
+    for (int j = 0; j < 5; ++j) {
+        const int d = 1 << j;
+        const float t1 = __shfl_up_sync(0xffffffffu, S1, d);
+        const float t2 = __shfl_up_sync(0xffffffffu, S2, d);
+        const float4 h = phi[j];
+        if (lane >= d) {
+            S1 = fmaf(h.x, t1, fmaf(h.y, t2, S1));
+            S2 = fmaf(h.z, t1, fmaf(h.w, t2, S2));
+        }
+    }
+    float q01 = __shfl_up_sync(0xffffffffu, S1, 1);
+    float q02 = __shfl_up_sync(0xffffffffu, S2, 1);
+    if (lane == 0) {
+        q01 = ST ? Z1 : 0.f;
+        q02 = C2;
+    }
+    const float q21 = fmaf(hp.x, q01, fmaf(hp.y, q02, A1));
+    const float q22 = fmaf(hp.z, q01, fmaf(hp.w, q02, A2));
+    const float q11 = fmaf(qp.x, q01, fmaf(qp.y, q02, s01));
+    const float q12 = fmaf(qp.z, q01, fmaf(qp.w, q02, s02));
+    const float q31 = fmaf(qp.x, q21, fmaf(qp.y, q22, s21));
+    const float q32 = fmaf(qp.z, q21, fmaf(qp.w, q22, s22));
+    // z2 = t s1 + w s2
+    const f2x pt = f2_dup(t), pw = f2_dup(cpl.x);
+    zu1 = f2_pack(q01, q11);
+    zw1 = f2_pack(q21, q31);
+    zu2 = f2_fma(pt, zu1, f2_mul(pw, f2_pack(q02, q12)));
+    zw2 = f2_fma(pt, zw1, f2_mul(pw, f2_pack(q22, q32)));
+}
+
+// One section over one group, from the group's incoming DF2T state (Z1, Z2)
+// (scaled by 1/G_k when b0 is factored); leaves the group's outgoing state in
+// (Z1, Z2).  The lane's chunk is filtered as four quarters side by side, two
+// packed chains of N/4 steps each from zero state; their outgoing states are
+// joined into the lane's by A^(N/4) (phi[6]) and A^(N/2) (phi[5]), the lane
+// states scanned, and the quarters re-run side by side from their true
+// incoming states.  What bounds it is the FMA pipe (6 FMAs per sample) once
+// the dependent chains and the scan are covered; measured alone (compute
+// only, 12 warps per SM, clock64), samples per clock and SM: one scalar chain
+// per lane 8.1 (N = 32), two half chunks packed 13.0 (N = 32) and 16.8
+// (N = 64), four quarters 14.3 and 20.0 -- 0.94 of the pipe at N = 64, where
+// one scan serves 2048 samples.
+// The states are joined, scanned and passed on in a basis of their own, s1 =
+// z1, s2 = (z2 - (a1/2) z1) / w (Coef32::cpl), in which A is a scaled rotation
+// (or symmetric) and no entry of its powers much exceeds 1: in the DF2T basis
+// they grow to about 1 / sin(pole angle) and the FP32 products cancel at every
+// step of the scan.
+// phi: the powers in that basis, Phi^(2^j), j = 0..4, A^(N/2), A^(N/4).
+// cpl: w, 1/w.  ZF: the group holds the channel's last sample (at element mq
+// of the chunk of the lane where zf_owner is set), whose DF2T state goes to
+// zf_dst; a separate instantiation, so that other groups carry none of it.
+// s_own: the lane's row (N floats, 16-byte aligned), scratch for ZF.
+// AL: the in-lane recursions add the low parts alo of a1, a2 (a section
+// whose poles FP32 coefficients would displace noticeably).
+template <int N, bool FACT, bool ZF = false, bool AL = false>
+__device__ __forceinline__ void pipe_section(QChunk<N>& v, const float4 ab, const float b0,
+                                             const float4* phi, const float2 cpl, float& Z1,
+                                             float& Z2, bool zf_owner, int mq, float* s_own,
+                                             float* zf_dst, float G, float2 alo = {0.f, 0.f}) {
+    constexpr int Q = N / 4;
+    const float b1 = ab.z, b2 = ab.w;
+    const f2x na1 = f2_dup(-ab.x), na2 = f2_dup(-ab.y), pb1 = f2_dup(b1), pb2 = f2_dup(b2);
+    const f2x nl1 = f2_dup(AL ? -alo.x : 0.f), nl2 = f2_dup(AL ? -alo.y : 0.f);
+    f2x(&u)[Q] = v.u;
+    f2x(&w)[Q] = v.w;
     // the all-pole terms, with a_i = ab + alo for AL (the low-part products
     // go first, into the smaller terms), FP32 a_i otherwise:
     // ap2 = t - a1 y1 - a2 y2, ap1 = t - a1 y1, st2 = -a1 y1 - a2 y2, st1 = -a2 y
-    auto ap2 = [&](float y1, float y2, float t) {
-        return fmaf(-a1, y1, fmaf(-a2, y2, AL ? fmaf(-alo.x, y1, fmaf(-alo.y, y2, t)) : t));
+    auto ap2 = [&](f2x y1, f2x y2, f2x t) {
+        return f2_fma(na1, y1, f2_fma(na2, y2, AL ? f2_fma(nl1, y1, f2_fma(nl2, y2, t)) : t));
     };
-    auto ap1 = [&](float y1, float t) { return fmaf(-a1, y1, AL ? fmaf(-alo.x, y1, t) : t); };
-    auto st2 = [&](float y1, float y2) {
-        return fmaf(-a1, y1, AL ? fmaf(-a2, y2, fmaf(-alo.x, y1, -alo.y * y2)) : -a2 * y2);
+    auto ap1 = [&](f2x y1, f2x t) { return f2_fma(na1, y1, AL ? f2_fma(nl1, y1, t) : t); };
+    auto st2 = [&](f2x y1, f2x y2) {
+        return f2_fma(na1, y1,
+                      AL ? f2_fma(na2, y2, f2_fma(nl1, y1, f2_mul(nl2, y2))) : f2_mul(na2, y2));
     };
-    auto st1 = [&](float y) { return AL ? fmaf(-a2, y, -alo.y * y) : -a2 * y; };
+    auto st1 = [&](f2x y) { return AL ? f2_fma(na2, y, f2_mul(nl2, y)) : f2_mul(na2, y); };
 
-    // S8 support: the section input at the channel's last sample (element mq
-    // of the owner's chunk), picked by compile-time-indexed selects
+    // S8 support: the section input at the channel's last sample
     float xq = 0.f, xqm1 = 0.f;
-    if (ZF) pick_pair<N>(v, mq, xq, xqm1);
+    if (ZF) pick_q<N>(v, mq, s_own, xq, xqm1);
 
+    // S3: non-recursive stage with zero history inside each quarter
+    const f2x ux1 = u[Q - 1], ux2 = u[Q - 2], wx1 = w[Q - 1], wx2 = w[Q - 2];
+    const f2x pb0 = f2_dup(b0);
+#pragma unroll
+    for (int m = Q - 1; m >= 2; --m) {
+        u[m] = f2_fma(pb2, u[m - 2], f2_fma(pb1, u[m - 1], FACT ? u[m] : f2_mul(pb0, u[m])));
+        w[m] = f2_fma(pb2, w[m - 2], f2_fma(pb1, w[m - 1], FACT ? w[m] : f2_mul(pb0, w[m])));
+    }
+    u[1] = f2_fma(pb1, u[0], FACT ? u[1] : f2_mul(pb0, u[1]));
+    w[1] = f2_fma(pb1, w[0], FACT ? w[1] : f2_mul(pb0, w[1]));
+    if (!FACT) {
+        u[0] = f2_mul(pb0, u[0]);
+        w[0] = f2_mul(pb0, w[0]);
+    }
+
+    // S4 (i): particular solutions from zero state, terminal values only
+    f2x p0 = u[0], p1 = ap1(p0, u[1]), r0 = w[0], r1 = ap1(r0, w[1]);
+#pragma unroll
+    for (int m = 2; m < Q; ++m) {
+        const f2x p2 = ap2(p1, p0, u[m]), r2 = ap2(r1, r0, w[m]);
+        p0 = p1;
+        p1 = p2;
+        r0 = r1;
+        r1 = r2;
+    }
+    // the quarters' zero-state outgoing states, and from them the quarters'
+    // incoming ones
+    const f2x e1u = f2_fma(pb1, ux1, f2_fma(pb2, ux2, st2(p1, p0)));
+    const f2x e2u = f2_fma(pb2, ux1, st1(p1));
+    const f2x e1w = f2_fma(pb1, wx1, f2_fma(pb2, wx2, st2(r1, r0)));
+    const f2x e2w = f2_fma(pb2, wx1, st1(r1));
+    f2x zu1, zu2, zw1, zw2;
+    join_states<true>(e1u, e2u, e1w, e2w, Z1, Z2, 0.5f * ab.x, cpl, phi, zu1, zu2, zw1, zw2);
+
+    // S4 (iii): re-run the recursions from the true incoming states
+    u[0] = f2_add(u[0], zu1);
+    w[0] = f2_add(w[0], zw1);
+    u[1] = ap1(u[0], f2_add(u[1], zu2));
+    w[1] = ap1(w[0], f2_add(w[1], zw2));
+#pragma unroll
+    for (int m = 2; m < Q; ++m) {
+        u[m] = ap2(u[m - 1], u[m - 2], u[m]);
+        w[m] = ap2(w[m - 1], w[m - 2], w[m]);
+    }
+
+    // the group's outgoing state, from lane 31's last two inputs and outputs
+    const float o1 = f2_b(f2_fma(pb1, wx1, f2_fma(pb2, wx2, st2(w[Q - 1], w[Q - 2]))));
+    const float o2 = f2_b(f2_fma(pb2, wx1, st1(w[Q - 1])));
+    Z1 = __shfl_sync(0xffffffffu, o1, 31);
+    Z2 = __shfl_sync(0xffffffffu, o2, 31);
+
+    // S8: final state at the channel's last sample
+    if (ZF) {
+        float yq, yqm1;
+        pick_q<N>(v, mq, s_own, yq, yqm1);
+        const f2x y1 = f2_dup(yq), y2 = f2_dup(yqm1);
+        float f1;
+        if (mq >= 1) f1 = fmaf(b1, xq, fmaf(b2, xqm1, f2_a(st2(y1, y2))));
+        else f1 = fmaf(b1, xq, f2_a(ap1(y1, zu2)));
+        const float f2 = fmaf(b2, xq, f2_a(st1(y1)));
+        if (zf_owner) {
+            zf_dst[0] = f1 * G;
+            zf_dst[1] = f2 * G;
+        }
+    }
+}
+
+// One section over one group with one scalar chain per lane, for the
+// backward's recomputation of the section signals: its gradient sums are held
+// to the rounding of this order of operations (the coefficient gradients of
+// cascades whose sections cancel each other amplify any other order's).
+// Arguments as above, FP32 throughout, no final state.
+// INJ: a DF2T state (zi1, zi2) enters at group-relative sample pinj instead
+// of the group start (the inputs before it being zero): added to the
+// all-pole input at pinj and pinj + 1 (a channel's first group, whose grid is
+// anchored elsewhere).
+template <int N, bool FACT, bool INJ>
+__device__ __forceinline__ void lane_section(float (&v)[N], const float4 ab, const float b0,
+                                             const float4* phi, const float4 lp, float& Z1,
+                                             float& Z2, int pinj = -1, float zi1 = 0.f,
+                                             float zi2 = 0.f) {
+    const int lane = threadIdx.x & 31;
+    const float a1 = ab.x, a2 = ab.y, b1 = ab.z, b2 = ab.w;
     // S3: non-recursive stage with zero history inside the lane
     const float xl1 = v[N - 1], xl2 = v[N - 2];
 #pragma unroll
@@ -105,98 +322,51 @@ __device__ __forceinline__ void pipe_section(float (&v)[N], const float4 ab, con
     }
 
     // S4 (i): particular solution from zero state, terminal values only
-    float w0 = v[0], w1 = ap1(w0, v[1]);
+    float w0 = v[0], w1 = fmaf(-a1, w0, v[1]);
 #pragma unroll
     for (int m = 2; m < N; ++m) {
-        const float w2 = ap2(w1, w0, v[m]);
+        const float w2 = fmaf(-a1, w1, fmaf(-a2, w0, v[m]));
         w0 = w1;
         w1 = w2;
     }
-    float S1 = fmaf(b1, xl1, fmaf(b2, xl2, st2(w1, w0)));
-    float S2 = fmaf(b2, xl1, st1(w1));
+    float S1 = fmaf(b1, xl1, fmaf(b2, xl2, fmaf(-a1, w1, -a2 * w0)));
+    float S2 = fmaf(b2, xl1, -a2 * w1);
 
-    float zin1, zin2;
-    if (DFS) {
-        // S4 (ii) and the fold in double-float; the chunk waits in the lane's
-        // row (s_own) meanwhile, so that its registers serve the scan
-        chunk_to_row<N>(v, s_own);
-        df s1 = df_from(S1), s2 = df_from(S2);
+    // S4 (ii): inclusive scan over lanes, z_{l+1} = Phi z_l + s_l
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int d = 1 << j;
-            df t1{__shfl_up_sync(0xffffffffu, s1.hi, d), __shfl_up_sync(0xffffffffu, s1.lo, d)};
-            df t2{__shfl_up_sync(0xffffffffu, s2.hi, d), __shfl_up_sync(0xffffffffu, s2.lo, d)};
-            if (lane < d) {
-                t1 = df_from(0.f);
-                t2 = df_from(0.f);
-            }
-            const float4 h = phi[j], l = phi_lo[j];
-            s1 = df_add_fast(s1, df_add_fast(df_mul(df{h.x, l.x}, t1), df_mul(df{h.y, l.y}, t2)));
-            s2 = df_add_fast(s2, df_add_fast(df_mul(df{h.z, l.z}, t1), df_mul(df{h.w, l.w}, t2)));
-        }
-        df e1{__shfl_up_sync(0xffffffffu, s1.hi, 1), __shfl_up_sync(0xffffffffu, s1.lo, 1)};
-        df e2{__shfl_up_sync(0xffffffffu, s2.hi, 1), __shfl_up_sync(0xffffffffu, s2.lo, 1)};
-        if (lane == 0) {
-            e1 = df_from(0.f);
-            e2 = df_from(0.f);
-        }
-        const df z1 = df_from(Z1), z2 = df_from(Z2);
-        zin1 = df_to_float(df_add_fast(
-            e1, df_add_fast(df_mul(df{lp.x, lpl.x}, z1), df_mul(df{lp.y, lpl.y}, z2))));
-        zin2 = df_to_float(df_add_fast(
-            e2, df_add_fast(df_mul(df{lp.z, lpl.z}, z1), df_mul(df{lp.w, lpl.w}, z2))));
-        row_to_chunk<N>(v, s_own);
-    } else {
-        // S4 (ii): inclusive scan over lanes, z_{l+1} = Phi z_l + s_l
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int d = 1 << j;
-            float t1 = __shfl_up_sync(0xffffffffu, S1, d);
-            float t2 = __shfl_up_sync(0xffffffffu, S2, d);
-            t1 = lane >= d ? t1 : 0.f;
-            t2 = lane >= d ? t2 : 0.f;
-            S1 = fmaf(phi[j].x, t1, fmaf(phi[j].y, t2, S1));
-            S2 = fmaf(phi[j].z, t1, fmaf(phi[j].w, t2, S2));
-        }
-        float E1 = __shfl_up_sync(0xffffffffu, S1, 1);
-        float E2 = __shfl_up_sync(0xffffffffu, S2, 1);
-        if (lane == 0) {
-            E1 = 0.f;
-            E2 = 0.f;
-        }
-        // fold the group's incoming state into this lane's: Phi^lane Z + E
-        zin1 = fmaf(lp.x, Z1, fmaf(lp.y, Z2, E1));
-        zin2 = fmaf(lp.z, Z1, fmaf(lp.w, Z2, E2));
+    for (int j = 0; j < 5; ++j) {
+        const int d = 1 << j;
+        float t1 = __shfl_up_sync(0xffffffffu, S1, d);
+        float t2 = __shfl_up_sync(0xffffffffu, S2, d);
+        t1 = lane >= d ? t1 : 0.f;
+        t2 = lane >= d ? t2 : 0.f;
+        S1 = fmaf(phi[j].x, t1, fmaf(phi[j].y, t2, S1));
+        S2 = fmaf(phi[j].z, t1, fmaf(phi[j].w, t2, S2));
     }
+    float E1 = __shfl_up_sync(0xffffffffu, S1, 1);
+    float E2 = __shfl_up_sync(0xffffffffu, S2, 1);
+    if (lane == 0) {
+        E1 = 0.f;
+        E2 = 0.f;
+    }
+    // fold the group's incoming state into this lane's: Phi^lane Z + E
+    const float zin1 = fmaf(lp.x, Z1, fmaf(lp.y, Z2, E1));
+    const float zin2 = fmaf(lp.z, Z1, fmaf(lp.w, Z2, E2));
 
     // S4 (iii): re-run the recursion from the true incoming state
     v[0] = v[0] + zin1;
-    v[1] = ap1(v[0], v[1] + zin2);
+    v[1] = fmaf(-a1, v[0], v[1] + zin2);
 #pragma unroll
-    for (int m = 2; m < N; ++m) v[m] = ap2(v[m - 1], v[m - 2], v[m]);
+    for (int m = 2; m < N; ++m) v[m] = fmaf(-a1, v[m - 1], fmaf(-a2, v[m - 2], v[m]));
 
     // the group's outgoing state, from lane 31's last two inputs and outputs
-    const float o1 = fmaf(b1, xl1, fmaf(b2, xl2, st2(v[N - 1], v[N - 2])));
-    const float o2 = fmaf(b2, xl1, st1(v[N - 1]));
+    const float o1 = fmaf(b1, xl1, fmaf(b2, xl2, fmaf(-a1, v[N - 1], -a2 * v[N - 2])));
+    const float o2 = fmaf(b2, xl1, -a2 * v[N - 1]);
     Z1 = __shfl_sync(0xffffffffu, o1, 31);
     Z2 = __shfl_sync(0xffffffffu, o2, 31);
     // a state injected at the group's last sample: its second component
     // belongs to the next group
     if (INJ && pinj == 32 * N - 1) Z1 += zi2;
-
-    // S8: final state at the channel's last sample
-    if (ZF) {
-        float yq, yqm1;
-        pick_pair<N>(v, mq, yq, yqm1);
-        float f1;
-        if (mq >= 1) f1 = fmaf(b1, xq, fmaf(b2, xqm1, st2(yq, yqm1)));
-        else f1 = fmaf(b1, xq, ap1(yq, zin2));
-        const float f2 = fmaf(b2, xq, st1(yq));
-        if (zf_owner) {
-            zf_dst[0] = f1 * G;
-            zf_dst[1] = f2 * G;
-        }
-    }
 }
 
 // Coefficients of one section in double-float, for channels run in extended
@@ -205,148 +375,250 @@ struct SecDF {
     df a1, a2, b0, b1, b2;
 };
 
-// One section over one group with the samples themselves in double-float:
-// the high parts in the lane's chunk vh[] (registers), the low parts in the
-// lane's row lo[] (shared memory, 16-byte aligned, read and written four at
-// a time, which the row padding makes bank-conflict free; registers would
-// double the section's footprint).  The same steps as pipe_section -- S3 with
-// zero in-lane history, S4 (i) the particular solution's terminal pair, (ii)
-// the lane scan and the fold of the group's incoming state, (iii) the re-run
-// from the true lane state, the group's outgoing state, S8 -- every one in
-// double-float (about 44 bits), so that neither the samples handed from
-// section to section nor the recursions' own roundings are limited to FP32.
-// For cascades in which later sections attenuate what earlier ones pass
-// (poles next to the unit circle), where FP32 rounding of an intermediate
-// signal reaches the output amplified many times.  Z1, Z2: the group's
-// incoming DF2T state, left outgoing.  ZF: the group holds the channel's last
-// sample (element mq of the chunk of the lane where zf_owner is set), whose
-// state goes to zf_dst.
+__device__ __forceinline__ f2x f2_neg1() { return f2_dup(-1.f); }
+
+// The all-pole solve of one group in FP32 (a_i = hi + lo parts): y_m = v_m -
+// a1 y_{m-1} - a2 y_{m-2} over the group from zero state, by quarters as in
+// pipe_section (particular solutions, joins, lane scan, re-run); y may be v.
+template <int N>
+__device__ __forceinline__ void pole_solve(const QChunk<N>& v, QChunk<N>& y, const f2x na1,
+                                           const f2x na2, const f2x nl1, const f2x nl2,
+                                           const float4* phi, const float2 cpl) {
+    constexpr int Q = N / 4;
+    auto ap2 = [&](f2x y1, f2x y2, f2x t) {
+        return f2_fma(na1, y1, f2_fma(na2, y2, f2_fma(nl1, y1, f2_fma(nl2, y2, t))));
+    };
+    auto ap1 = [&](f2x y1, f2x t) { return f2_fma(na1, y1, f2_fma(nl1, y1, t)); };
+    f2x p0 = v.u[0], p1 = ap1(p0, v.u[1]), r0 = v.w[0], r1 = ap1(r0, v.w[1]);
+#pragma unroll
+    for (int m = 2; m < Q; ++m) {
+        const f2x p2 = ap2(p1, p0, v.u[m]), r2 = ap2(r1, r0, v.w[m]);
+        p0 = p1;
+        p1 = p2;
+        r0 = r1;
+        r1 = r2;
+    }
+    f2x zu1, zu2, zw1, zw2;
+    join_states<false>(f2_fma(na1, p1, f2_mul(na2, p0)), f2_mul(na2, p1),
+                       f2_fma(na1, r1, f2_mul(na2, r0)), f2_mul(na2, r1), 0.f, 0.f,
+                       -0.5f * f2_a(na1), cpl, phi, zu1, zu2, zw1, zw2);
+    y.u[0] = f2_add(v.u[0], zu1);
+    y.w[0] = f2_add(v.w[0], zw1);
+    y.u[1] = ap1(y.u[0], f2_add(v.u[1], zu2));
+    y.w[1] = ap1(y.w[0], f2_add(v.w[1], zw2));
+#pragma unroll
+    for (int m = 2; m < Q; ++m) {
+        y.u[m] = ap2(y.u[m - 1], y.u[m - 2], v.u[m]);
+        y.w[m] = ap2(y.w[m - 1], y.w[m - 2], v.w[m]);
+    }
+}
+
+// The values at m = -j (j = 1, 2) of both pairs of quarters: quarter q's are
+// the last of quarter q - 1, the first quarter's the previous lane's (zero
+// for lane 0).
+template <int N>
+__device__ __forceinline__ void q_history(const QChunk<N>& v, int j, f2x& hu, f2x& hw) {
+    constexpr int Q = N / 4;
+    float ua, ub, wa, wb;
+    f2_unpack(v.u[Q - j], ua, ub);
+    f2_unpack(v.w[Q - j], wa, wb);
+    float prev = __shfl_up_sync(0xffffffffu, wb, 1);
+    if ((threadIdx.x & 31) == 0) prev = 0.f;
+    hu = f2_pack(prev, ua);
+    hw = f2_pack(ub, wa);
+}
+
+template <int N>
+__device__ __forceinline__ float q_max(const QChunk<N>& v) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < N / 4; ++i) {
+        float a, b, c, d;
+        f2_unpack(v.u[i], a, b);
+        f2_unpack(v.w[i], c, d);
+        m = fmaxf(fmaxf(m, fmaxf(fabsf(a), fabsf(b))), fmaxf(fabsf(c), fabsf(d)));
+    }
+    return m;
+}
+
+// 1.5 * 2^e such that sums of terms up to `bound` in absolute value, added to
+// it one by one, stay in its binade (then each addition's rounding error is
+// itself an FP32 number, recovered by two more operations).
+__device__ __forceinline__ float sum_anchor(float bound) {
+    const int e = min((__float_as_int(bound) >> 23) & 0xff, 251) + 2;
+    return __int_as_float((e << 23) | 0x400000);
+}
+
+// One section over one group with the samples in double-float (about 44
+// bits): hi and lo parts in registers, for cascades in which later sections
+// attenuate what earlier ones pass (poles next to the unit circle), where FP32
+// rounding of an intermediate signal reaches the output amplified many times.
+// The section's banded system is solved by iterative refinement (Wilkinson;
+// Higham, Accuracy and Stability of Numerical Algorithms, ch. 12): its
+// right-hand side, the FIR's output, is formed to about 2^-46 of its terms;
+// an FP32 solve (pole_solve) gives y0; the residual u - A y0 is formed to the
+// same 2^-46, where its terms cancel; a second FP32 solve gives the
+// correction, and y = y0 + correction as hi and lo parts.  Each round divides
+// the error by the FP32 solve's own relative error, and the rounding of y0
+// needs no compensated recursion: every chain of dependent steps is an FP32
+// one, and the long sums are independent from sample to sample and packed.
+// (Solving the recursions step by step in double-float takes about 27
+// dependent operations per sample, twice, and a double-float scan; 64 channels
+// of 2^22 samples, K = 8, half of them in double-float: 32.6 ms that way, 14.5
+// this way.)
+// The long sums add their products one by one to an anchor far larger than
+// the sum (sum_anchor): each addition's error comes back exactly from two
+// more FMAs, and the errors are summed beside the low parts.
+// xh, xl: the section's input, replaced by its output.  mx: max |x| of the
+// lane, replaced by max |y|.  Z1, Z2: the group's incoming DF2T state in
+// double-float, left outgoing.  refine: rounds of refinement.  ZF: the group
+// holds the channel's last sample (element mq of the chunk of the lane where
+// zf_owner is set), whose state goes to zf_dst; row: scratch for it.
 template <int N, bool ZF = false>
-__device__ __forceinline__ void pipe_section_dfx(float (&vh)[N], float* lo, const SecDF& q,
-                                                 const float4* phi, const float4* phi_lo,
-                                                 const float4 lp, const float4 lpl, df& Z1,
-                                                 df& Z2, bool zf_owner, int mq, float* zf_dst) {
+__device__ __forceinline__ void pipe_section_dfx(QChunk<N>& xh, QChunk<N>& xl, float& mx,
+                                                 const SecDF& q, const float4* phi,
+                                                 const float2 cpl, int refine, df& Z1, df& Z2, bool zf_owner, int mq, float* row,
+                                                 float* zf_dst) {
+    constexpr int Q = N / 4;
     const int lane = threadIdx.x & 31;
-    const df na1 = df_neg(q.a1);
-    float4* lo4 = reinterpret_cast<float4*>(lo);
-    df xq{0.f, 0.f}, xqm1{0.f, 0.f};
+    const f2x m1 = f2_neg1();
+    // c += the rounding error of t = T + b x, T <- t
+    auto term = [&](f2x b, f2x x, f2x& T, f2x& c) {
+        const f2x t = f2_fma(b, x, T);
+        c = f2_add(c, f2_fma(b, x, f2_fma(t, m1, T)));
+        T = t;
+    };
+    // the same for t = T + v
+    auto term1 = [&](f2x v, f2x& T, f2x& c) {
+        const f2x t = f2_add(v, T);
+        c = f2_add(c, f2_add(v, f2_fma(t, m1, T)));
+        T = t;
+    };
+    df xq{0.f, 0.f}, xqm1{0.f, 0.f}, xp1{0.f, 0.f};
     if (ZF) {
-        pick_pair<N>(vh, mq, xq.hi, xqm1.hi);
-        xq.lo = lo[mq];
-        xqm1.lo = mq >= 1 ? lo[mq - 1] : 0.f;
+        pick_q<N>(xh, mq, row, xq.hi, xqm1.hi);
+        pick_q<N>(xl, mq, row, xq.lo, xqm1.lo);
+        xp1.hi = __shfl_up_sync(0xffffffffu, f2_b(xh.w[Q - 1]), 1);
+        xp1.lo = __shfl_up_sync(0xffffffffu, f2_b(xl.w[Q - 1]), 1);
     }
-    const float4 top = lo4[N / 4 - 1];
-    const df xl1{vh[N - 1], top.w}, xl2{vh[N - 2], top.z};
-    // S3, top down (block q of four samples reads the inputs of blocks q and
-    // q - 1, which the steps below it have not overwritten yet)
+    // the inputs that the outgoing state is formed from
+    const df xe1{f2_b(xh.w[Q - 1]), f2_b(xl.w[Q - 1])}, xe2{f2_b(xh.w[Q - 2]), f2_b(xl.w[Q - 2])};
+
+    // S3 in double-float: u = b0 x + b1 x' + b2 x'', plus the group's state on
+    // its first two samples; in place, top down
+    float mu;
+    {
+        const float cb = fabsf(q.b0.hi) + fabsf(q.b1.hi) + fabsf(q.b2.hi);
+        mu = fmaxf(mx, __shfl_up_sync(0xffffffffu, mx, 1)) * cb;
+        if (lane == 0) mu += fabsf(Z1.hi) + fabsf(Z2.hi);
+        mu *= 1.001f;
+        const f2x M = f2_dup(sum_anchor(mu));
+        const f2x b0 = f2_dup(q.b0.hi), b1 = f2_dup(q.b1.hi), b2 = f2_dup(q.b2.hi);
+        const f2x l0 = f2_dup(q.b0.lo), l1 = f2_dup(q.b1.lo), l2 = f2_dup(q.b2.lo);
+        f2x hu1, hw1, hu2, hw2, gu1, gw1, gu2, gw2;
+        q_history<N>(xh, 1, hu1, hw1);
+        q_history<N>(xh, 2, hu2, hw2);
+        q_history<N>(xl, 1, gu1, gw1);
+        q_history<N>(xl, 2, gu2, gw2);
+        auto fir = [&](f2x& h0, f2x& g0, f2x h1, f2x g1, f2x h2, f2x g2, f2x zh, f2x zl, bool z) {
+            f2x T = f2_fma(b0, h0, M);
+            f2x c = f2_fma(b0, h0, f2_fma(T, m1, M));
+            term(b1, h1, T, c);
+            term(b2, h2, T, c);
+            if (z) {
+                term1(zh, T, c);
+                c = f2_add(c, zl);
+            }
+            c = f2_fma(b0, g0, f2_fma(l0, h0, c));
+            c = f2_fma(b1, g1, f2_fma(l1, h1, c));
+            c = f2_fma(b2, g2, f2_fma(l2, h2, c));
+            h0 = f2_fma(M, m1, T);
+            g0 = c;
+        };
+        const bool l0z = lane == 0;
+        const f2x zh1 = f2_pack(l0z ? Z1.hi : 0.f, 0.f), zl1 = f2_pack(l0z ? Z1.lo : 0.f, 0.f);
+        const f2x zh2 = f2_pack(l0z ? Z2.hi : 0.f, 0.f), zl2 = f2_pack(l0z ? Z2.lo : 0.f, 0.f);
 #pragma unroll
-    for (int b = N / 4 - 1; b >= 0; --b) {
-        const float4 c = lo4[b];
-        const float4 d = b > 0 ? lo4[b > 0 ? b - 1 : 0] : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float l[6] = {d.z, d.w, c.x, c.y, c.z, c.w};  // lo of x_{4b-2} .. x_{4b+3}
-        float h[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            const int m = 4 * b - 2 + i;
-            h[i] = m >= 0 ? vh[m >= 0 ? m : 0] : 0.f;
+        for (int m = Q - 1; m >= 2; --m) {
+            fir(xh.u[m], xl.u[m], xh.u[m - 1], xl.u[m - 1], xh.u[m - 2], xl.u[m - 2], 0, 0, false);
+            fir(xh.w[m], xl.w[m], xh.w[m - 1], xl.w[m - 1], xh.w[m - 2], xl.w[m - 2], 0, 0, false);
         }
-        float out[4];
-#pragma unroll
-        for (int i = 3; i >= 0; --i) {
-            const int m = 4 * b + i;
-            df u;
-            if (m >= 2)
-                u = df_dot3(q.b0, df{h[i + 2], l[i + 2]}, q.b1, df{h[i + 1], l[i + 1]}, q.b2,
-                            df{h[i], l[i]});
-            else if (m == 1)
-                u = df_dot3(q.b0, df{h[i + 2], l[i + 2]}, q.b1, df{h[i + 1], l[i + 1]},
-                            df{0.f, 0.f}, df{0.f, 0.f});
-            else
-                u = df_mul(q.b0, df{h[i + 2], l[i + 2]});
-            vh[m] = u.hi;
-            out[i] = u.lo;
-        }
-        lo4[b] = make_float4(out[0], out[1], out[2], out[3]);
+        fir(xh.u[1], xl.u[1], xh.u[0], xl.u[0], hu1, gu1, zh2, zl2, true);
+        fir(xh.w[1], xl.w[1], xh.w[0], xl.w[0], hw1, gw1, 0, 0, false);
+        fir(xh.u[0], xl.u[0], hu1, gu1, hu2, gu2, zh1, zl1, true);
+        fir(xh.w[0], xl.w[0], hw1, gw1, hw2, gw2, 0, 0, false);
     }
-    // S4 (i): the particular solution from zero state, its terminal pair
-    df w0{0.f, 0.f}, w1{0.f, 0.f};
+
+    // S4: the FP32 solve, then refinement; xh, xl hold the right-hand side
+    const f2x na1 = f2_dup(-q.a1.hi), na2 = f2_dup(-q.a2.hi);
+    const f2x nl1 = f2_dup(-q.a1.lo), nl2 = f2_dup(-q.a2.lo);
+    QChunk<N> y, d;
+    pole_solve<N>(xh, y, na1, na2, nl1, nl2, phi, cpl);
+    mx = q_max<N>(y);
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+        const float my = fmaxf(mx, __shfl_up_sync(0xffffffffu, mx, 1));
+        const f2x M = f2_dup(sum_anchor(1.001f * fmaf(4.f, my, mu)));
+        f2x hu1, hw1, hu2, hw2;
+        q_history<N>(y, 1, hu1, hw1);
+        q_history<N>(y, 2, hu2, hw2);
+        auto res = [&](f2x h, f2x g, f2x y0, f2x y1, f2x y2) -> f2x {
+            f2x T = f2_add(h, M);
+            f2x c = f2_add(g, f2_add(h, f2_fma(T, m1, M)));
+            term(na1, y1, T, c);
+            term(na2, y2, T, c);
+            term(m1, y0, T, c);
+            c = f2_fma(nl1, y1, f2_fma(nl2, y2, c));
+            return f2_add(f2_fma(M, m1, T), c);
+        };
 #pragma unroll
-    for (int b = 0; b < N / 4; ++b) {
-        const float4 c = lo4[b];
-        const float l[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int m = 4 * b + i;
-            const df u{vh[m], l[i]};
-            df w2;
-            if (m == 0) w2 = u;
-            else if (m == 1) w2 = df_rec1(u, q.a1, w1);
-            else w2 = df_rec(u, q.a1, w1, q.a2, w0);
-            w0 = w1;
-            w1 = w2;
+        for (int m = 0; m < Q; ++m) {
+            d.u[m] = res(xh.u[m], xl.u[m], y.u[m], m >= 1 ? y.u[m >= 1 ? m - 1 : 0] : hu1,
+                         m >= 2 ? y.u[m >= 2 ? m - 2 : 0] : (m == 1 ? hu1 : hu2));
+            d.w[m] = res(xh.w[m], xl.w[m], y.w[m], m >= 1 ? y.w[m >= 1 ? m - 1 : 0] : hw1,
+                         m >= 2 ? y.w[m >= 2 ? m - 2 : 0] : (m == 1 ? hw1 : hw2));
         }
-    }
-    df s1 = df_rec1(df_dot3(q.b1, xl1, q.b2, xl2, na1, w1), q.a2, w0);
-    df s2 = df_rec1(df_mul(q.b2, xl1), q.a2, w1);
-    // S4 (ii): lane scan, z_{l+1} = Phi z_l + s_l, in double-float
+        pole_solve<N>(d, d, na1, na2, nl1, nl2, phi, cpl);
+        if (it + 1 >= refine) break;
+        // another round from the corrected solution, rounded
 #pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        const int d = 1 << j;
-        df t1{__shfl_up_sync(0xffffffffu, s1.hi, d), __shfl_up_sync(0xffffffffu, s1.lo, d)};
-        df t2{__shfl_up_sync(0xffffffffu, s2.hi, d), __shfl_up_sync(0xffffffffu, s2.lo, d)};
-        if (lane < d) {
-            t1 = df{0.f, 0.f};
-            t2 = df{0.f, 0.f};
+        for (int m = 0; m < Q; ++m) {
+            y.u[m] = f2_add(y.u[m], d.u[m]);
+            y.w[m] = f2_add(y.w[m], d.w[m]);
         }
-        const float4 h = phi[j], l = phi_lo[j];
-        s1 = df_add(s1, df_add(df_mul(df{h.x, l.x}, t1), df_mul(df{h.y, l.y}, t2)));
-        s2 = df_add(s2, df_add(df_mul(df{h.z, l.z}, t1), df_mul(df{h.w, l.w}, t2)));
+        mx = q_max<N>(y);
     }
-    df e1{__shfl_up_sync(0xffffffffu, s1.hi, 1), __shfl_up_sync(0xffffffffu, s1.lo, 1)};
-    df e2{__shfl_up_sync(0xffffffffu, s2.hi, 1), __shfl_up_sync(0xffffffffu, s2.lo, 1)};
-    if (lane == 0) {
-        e1 = df{0.f, 0.f};
-        e2 = df{0.f, 0.f};
+    // y + d as hi and lo parts
+#pragma unroll
+    for (int m = 0; m < Q; ++m) {
+        xh.u[m] = f2_add(y.u[m], d.u[m]);
+        xl.u[m] = f2_add(d.u[m], f2_fma(xh.u[m], m1, y.u[m]));
+        xh.w[m] = f2_add(y.w[m], d.w[m]);
+        xl.w[m] = f2_add(d.w[m], f2_fma(xh.w[m], m1, y.w[m]));
     }
-    // fold the group's incoming state into this lane's: Phi^lane Z + E
-    const df zin1 = df_add(e1, df_add(df_mul(df{lp.x, lpl.x}, Z1), df_mul(df{lp.y, lpl.y}, Z2)));
-    const df zin2 = df_add(e2, df_add(df_mul(df{lp.z, lpl.z}, Z1), df_mul(df{lp.w, lpl.w}, Z2)));
-    // S4 (iii): the re-run from the true lane state
-    df y1{0.f, 0.f}, y2{0.f, 0.f};  // y_{m-1}, y_{m-2}
-#pragma unroll
-    for (int b = 0; b < N / 4; ++b) {
-        const float4 c = lo4[b];
-        const float l[4] = {c.x, c.y, c.z, c.w};
-        float out[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int m = 4 * b + i;
-            const df u{vh[m], l[i]};
-            df y;
-            if (m == 0) y = df_add(u, zin1);
-            else if (m == 1) y = df_rec1(df_add(u, zin2), q.a1, y1);
-            else y = df_rec(u, q.a1, y1, q.a2, y2);
-            vh[m] = y.hi;
-            out[i] = y.lo;
-            y2 = y1;
-            y1 = y;
-        }
-        lo4[b] = make_float4(out[0], out[1], out[2], out[3]);
+
+    // S8 support: the state's second component entering this lane
+    df zin2{0.f, 0.f};
+    const df na1d = df_neg(q.a1);
+    if (ZF) {
+        const df yp{__shfl_up_sync(0xffffffffu, f2_b(xh.w[Q - 1]), 1),
+                    __shfl_up_sync(0xffffffffu, f2_b(xl.w[Q - 1]), 1)};
+        zin2 = lane == 0 ? Z2 : df_rec1(df_mul(q.b2, xp1), q.a2, yp);
     }
     // the group's outgoing state, from lane 31's last two inputs and outputs
-    const df o1 = df_rec1(df_dot3(q.b1, xl1, q.b2, xl2, na1, y1), q.a2, y2);
-    const df o2 = df_rec1(df_mul(q.b2, xl1), q.a2, y1);
+    const df ye1{f2_b(xh.w[Q - 1]), f2_b(xl.w[Q - 1])}, ye2{f2_b(xh.w[Q - 2]), f2_b(xl.w[Q - 2])};
+    const df o1 = df_rec1(df_dot3(q.b1, xe1, q.b2, xe2, na1d, ye1), q.a2, ye2);
+    const df o2 = df_rec1(df_mul(q.b2, xe1), q.a2, ye1);
     Z1 = df{__shfl_sync(0xffffffffu, o1.hi, 31), __shfl_sync(0xffffffffu, o1.lo, 31)};
     Z2 = df{__shfl_sync(0xffffffffu, o2.hi, 31), __shfl_sync(0xffffffffu, o2.lo, 31)};
     // S8: final state at the channel's last sample
     if (ZF) {
         df yq, yqm1;
-        pick_pair<N>(vh, mq, yq.hi, yqm1.hi);
-        yq.lo = lo[mq];
-        yqm1.lo = mq >= 1 ? lo[mq - 1] : 0.f;
+        pick_q<N>(xh, mq, row, yq.hi, yqm1.hi);
+        pick_q<N>(xl, mq, row, yq.lo, yqm1.lo);
         df f1;
-        if (mq >= 1) f1 = df_rec1(df_dot3(q.b1, xq, q.b2, xqm1, na1, yq), q.a2, yqm1);
-        else f1 = df_add(df_dot3(q.b1, xq, na1, yq, df{0.f, 0.f}, df{0.f, 0.f}), zin2);
+        if (mq >= 1) f1 = df_rec1(df_dot3(q.b1, xq, q.b2, xqm1, na1d, yq), q.a2, yqm1);
+        else f1 = df_add(df_dot3(q.b1, xq, na1d, yq, df{0.f, 0.f}, df{0.f, 0.f}), zin2);
         const df f2 = df_rec1(df_mul(q.b2, xq), q.a2, yq);
         if (zf_owner) {
             zf_dst[0] = df_to_float(f1);

@@ -39,15 +39,21 @@ __device__ __forceinline__ float4 to_f4(const dfm2& m) {
     return make_float4(df_to_float(m.a), df_to_float(m.b), df_to_float(m.c), df_to_float(m.d));
 }
 
-// what to_f4 dropped: x - to_f4(x) per entry, the low word of the stored
-// double-float power
-__device__ __forceinline__ float df_rest(df x) {
-    const float h = df_to_float(x);
-    return (x.hi - h) + x.lo;
+// The scan's basis (Coef32::phi_c): its scale w, and a power of A in it,
+// T^-1 R T with T = [[1, 0], [a1/2, w]].
+__device__ __forceinline__ float scan_scale(double a1, double a2) {
+    const double disc = fma(0.25 * a1, a1, -a2);
+    const float sq = sqrtf(fabsf((float)disc));
+    const float r = disc < 0.0 ? sqrtf((float)a2) : 0.5f * fabsf((float)a1) + sq;
+    return fmaxf(fmaxf(sq, fabsf(1.f - r)), 0x1p-20f);
 }
 
-__device__ __forceinline__ float4 to_f4_lo(const dfm2& m) {
-    return make_float4(df_rest(m.a), df_rest(m.b), df_rest(m.c), df_rest(m.d));
+__device__ __forceinline__ float4 scan_basis(const dfm2& R, double a1, float w) {
+    const df t = df_of_double(0.5 * a1);
+    const df p11 = df_add(R.a, df_mul(R.b, t));
+    const df p21 = df_add(df_add(R.c, df_mul(R.d, t)), df_neg(df_mul(t, p11)));
+    return make_float4(df_to_float(p11), df_to_float(df_mul(R.b, df_from(w))),
+                       df_to_float(p21) / w, df_to_float(df_add(R.d, df_neg(df_mul(t, R.b)))));
 }
 
 __device__ __forceinline__ float max_entry(const dfm2& m) {
@@ -554,15 +560,16 @@ __device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int& t
 }
 
 // The horizon from the per-pole terms and ||h||_2 >= h2 (the pole warp), and
-// the channel's segment length: the call's T, or longer when the horizon
-// needs it (a segment is at least 2 P and long enough for the initial
+// the channel's tile length: the call's T, or longer when the horizon
+// needs it (a tile is at least 2 P and long enough for the initial
 // state's response to decay below the bound, rounded up to whole groups of
 // G), so that long-memory channels keep a bounded warm-up instead of being
-// carried; minseg, the shortest segment the horizon allows.  -1 where no
-// horizon holds.
+// carried; minseg, the shortest segment the horizon allows; zdecay, the
+// samples an initial state's response takes to decay (at least P).  -1 where
+// no horizon holds.
 __device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, float la, float ilr,
                                float zs, float lr, int64_t& seg, int32_t& minseg,
-                               int32_t& minseg_z) {
+                               int32_t& minseg_z, int32_t& zdecay) {
     float ptail = ilr != 0.f ? (la + __logf(h2)) * ilr : 0.f;
     // the initial state's response (each pole's share counted 2K times) has
     // decayed below the bound after tz samples
@@ -583,9 +590,40 @@ __device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, f
     // channel, and past an initial state's response (the streaming mode's
     // segments, where latency, not the warm-up's share, is what counts)
     const int64_t least = P > itz ? P : itz;
+    zdecay = (int32_t)least;
     minseg = (int32_t)((P + G - 1) / G * G > G ? (P + G - 1) / G * G : G);
     minseg_z = (int32_t)((least + G - 1) / G * G > G ? (least + G - 1) / G * G : G);
     return (int)P;
+}
+
+// The warp-segment kernel's segments of a channel of memory horizon P and
+// precision class e.  A warp's time goes with its warm-up and its outputs, S +
+// P, and the call is over when its slowest warp is, so:
+//  - S starts from the call's samples per resident warp (Params::wseg, whole
+//    groups, at most 64): one round of segments for a call that the GPU holds
+//    at once, however small (8,192 samples, K = 1: four warps of two groups
+//    each take 8 us, one warp of four 11);
+//  - double-float sections cost several times the FP32 ones: a quarter of it;
+//  - where 2 P is longer, S grows towards 2 P (a warm-up of half the outputs)
+//    as long as S + P stays below a few times the samples per warp, so that
+//    the channels with the longest memory do not end long after the others
+//    (64 channels of 2^22 samples, P = 43K..270K: 14.5 ms against 15.1
+//    with 2 P; 16 channels of 100,003, P = 4416: 88 us against 155), but not
+//    below P/4.
+// S + P is then rounded up to whole groups: the last one is computed anyway.
+__device__ __forceinline__ void warp_segments(const Params& p, int c, int64_t len, int64_t P,
+                                              int e) {
+    const int64_t G = 32LL * (e >= 3 ? ext_n(p.N) : p.N);
+    int64_t S = e >= 3 ? (p.wseg + 3) / 4 : p.wseg;
+    if (2 * P > S) {
+        int64_t want = (e >= 3 ? 3 : 2) * p.fair - P;
+        const int64_t least = S > P / 4 ? S : P / 4;
+        want = want < 2 * P ? want : 2 * P;
+        S = want > least ? want : least;
+    }
+    S = (S + P + G - 1) / G * G - P;
+    p.chan[c].seg = S;
+    p.chan[c].nseg = len > 0 ? (int32_t)((len + S - 1) / S) : 0;
 }
 
 // Block C: the channel table.
@@ -657,6 +695,11 @@ __device__ __forceinline__ void plan_table(const Params& p) {
     }
 }
 
+// Params::fair as kept in the plan cache's call-level key (wseg follows from it)
+__device__ __forceinline__ int32_t key_fair(const Params& p) {
+    return p.fair < 0x7fffffff ? (int32_t)p.fair : 0x7fffffff;
+}
+
 // Block c < C: the coefficient tables and the memory horizon of channel c.
 // Returns false when the channel's tables were kept from the previous plan on
 // this workspace (plan cache: same raw sos rows bit for bit, same K and
@@ -690,6 +733,8 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
     __shared__ cpx s_pole2[2 * kMaxSections];  // the precision warp's copy
     // [0..4] Phi^(2^j); [5..9] Psi^(2^r); [10..19] Theta^(2^i)
     __shared__ dfm2 s_chain[kMaxSections][20];
+    __shared__ dfm2 s_part[kMaxSections][3];  // A^(N/2), A^(N/4), A^(N/8)
+    __shared__ int s_ext;
 
     const int k = warp;
     // the section's row is read before K is known (one memory round trip, not
@@ -726,12 +771,12 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         const WsHeader* h = p.hdr;
         const int32_t hv = h->key_valid, hN = h->key_N, hW = h->key_W, ha = h->key_algo,
                       hf = h->key_flags, hk = h->key_kmax, hC = h->key_C;
-        const int64_t hs = h->key_seg, hc = h->key_cap;
+        const int64_t hs = h->key_seg, hc = h->key_cap, hfair = h->key_fair;
         const int32_t kv = kh->valid, kK = kh->K;
         const int64_t kl = kh->len, len = p.lengths[c];
         const bool same = !(p.flags_opt & SOS_FLAG_REPLAN) & (hv == 1) & (hN == p.N) &
                           (hW == p.W) & (ha == p.algo) & (hf == p.flags_opt) & (hk == kmax) &
-                          (hC == p.C) & (hs == p.seg) & (hc == p.cap_tiles) & (kv == 1) &
+                          (hC == p.C) & (hs == p.seg) & (hfair == key_fair(p)) & (hc == p.cap_tiles) & (kv == 1) &
                           (kK == K) & (kl == len);
         s_same[kMaxSections] = same;
     }
@@ -834,10 +879,10 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         // conditioned (slow-building responses of poles near the unit circle)
         const float h2 = fmaxf(s_h2, 0.5f * sqrtf(etail));
         int64_t seg = p.seg;
-        int32_t minseg = 0, minseg_z = 0;
+        int32_t minseg = 0, minseg_z = 0, zdecay = 0;
         int P = carry_only ? -1
                            : horizon_combine(ok, h2, Kc, p.seg, 32LL * p.N, la, ilr, zs, lr, seg,
-                                             minseg, minseg_z);
+                                             minseg, minseg_z, zdecay);
         // a channel without a partial-fraction horizon (repeated poles)
         // takes the cruder bound: always in backward plans, which have no
         // look-back (so that it is still cut into segments, warm-ups of P on
@@ -855,6 +900,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
                 P = Pf;
                 seg = p.seg;
                 if (want > seg) seg = (want + G - 1) / G * G;
+                zdecay = tzf > Pf ? tzf : Pf;
                 minseg = (int32_t)((Pf + G - 1) / G * G > G ? (Pf + G - 1) / G * G : G);
                 minseg_z = (int32_t)((tzf + G - 1) / G * G > minseg ? (tzf + G - 1) / G * G
                                                                      : minseg);
@@ -863,7 +909,10 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         // and a channel with no horizon at all is one segment, run from its
         // start to its end by one pipeline
         const int single = (P < 0 && (p.flags_opt & kFlagBackwardPlan)) ? 1 : 0;
-        if (single) P = 0;
+        if (single) {
+            P = 0;
+            zdecay = 0;
+        }
         if (lane == 0) {
             int64_t len = p.lengths[c];
             if (len < 0) len = 0;
@@ -876,6 +925,10 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
             p.chan[c].single = (int16_t)single;
             if (Kc == 0) p.chan[c].ext = 0;  // (else written by the first section warp)
             p.chan[c].seg = P >= 0 ? seg : p.seg;
+            p.chan[c].nseg = (int32_t)nt;
+            p.chan[c].zdecay = zdecay;
+            if (P >= 0 && Kc == 0 && !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE)))
+                warp_segments(p, c, len, P, 0);  // (else by the first section warp)
             p.chan[c].minseg = P >= 0 ? minseg : 0;
             p.chan[c].minseg_z = P >= 0 ? minseg_z : 0;
             p.chan[c].ntiles = (int32_t)nt;
@@ -910,7 +963,12 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         const dfm2 A{df_of_double(-a1), df{1.f, 0.f}, df_of_double(-a2), df{0.f, 0.f}};
         dfm2 P = A;
         // (exact additions: Phi^16 also seeds the look-back's tile powers)
-        for (int n = 1; n < N; n <<= 1) P = dfm_mul(P, P);  // A^N (N a power of two)
+        for (int n = 1; n < N; n <<= 1) {  // A^N (N a power of two)
+            if (2 * n == N) s_part[k][0] = P;  // A^(N/2), A^(N/4): half and quarter chunks
+            if (4 * n == N) s_part[k][1] = P;
+            if (8 * n == N) s_part[k][2] = P;
+            P = dfm_mul(P, P);
+        }
         s_chain[k][0] = P;
         for (int j = 1; j < 5; ++j) {
             P = dfm_mul(P, P);
@@ -964,13 +1022,20 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         for (int j = 0; j < 5; ++j)
             if ((lane >> j) & 1) P = dfm_mul(P, s_chain[k][j]);
         out32->lane_pow[lane] = to_f4(P);
-        out32->lane_lo[lane] = to_f4_lo(P);
+        // (at N = 64 over the powers of A^32, so that a channel's precision
+        // class is that of N = 32)
         m = max_entry(P);
+        if (ext_n(N) != N) m = lane < 16 ? fmaxf(m, max_entry(dfm_mul(P, s_part[k][0]))) : 0.f;
         if (lane < 5) {
             const dfm2 Q = s_chain[k][lane];
             out32->phi_pow[lane] = to_f4(Q);
-            out32->phi_lo[lane] = to_f4_lo(Q);
-            m = fmaxf(m, max_entry(Q));
+            if (ext_n(N) == N) m = fmaxf(m, max_entry(Q));
+        }
+        if (lane < 7) {
+            const float w = scan_scale(a1, a2);
+            out32->phi_c[lane] =
+                scan_basis(lane < 5 ? s_chain[k][lane] : s_part[k][lane - 5], a1, w);
+            if (lane == 0) out32->cpl = make_float4(w, 1.f / w, 0.f, 0.f);
         }
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
@@ -1029,8 +1094,25 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         p.chan[c].ext = e;
         p.chan[c].dflo = (int16_t)(e == 3 ? lo : 0);
         p.chan[c].dfhi = (int16_t)(e == 3 ? hi : Kc - 1);
+        s_ext = e;
+        if (s_horizon >= 0 &&
+            !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE)))
+            warp_segments(p, c, p.lengths[c], s_horizon, e);
     }
-    if (s_horizon >= 0) return true;
+    if (s_horizon >= 0) {
+        if (ext_n(N) != N &&
+            !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE))) {
+            // a channel of precision class 3 runs with ext_n(N) = N/2 samples
+            // per lane: its powers again, one squaring earlier
+            asm volatile("bar.sync 4, %0;" ::"r"(32 * Kc) : "memory");
+            if (s_ext >= 3 && lane < 7)
+                out32->phi_c[lane] = scan_basis(lane == 0   ? s_part[k][0]
+                                                : lane < 5 ? s_chain[k][lane - 1]
+                                                           : s_part[k][lane - 4],
+                                                a1, scan_scale(a1, a2));
+        }
+        return true;
+    }
     if (lane == 0) {
         dfm2 P = dfm_mul(s_chain[k][4], s_chain[k][4]);  // Psi = Phi^32
         s_chain[k][5] = P;
@@ -1096,9 +1178,9 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
     __shared__ int64_t s_wsum[32];
     // ---- prefixes: look-back tiles of the carried channels (tb, by
     // channel) and segments of the channels within their horizon (tbp, by
-    // dispatch position: porder lists the channels run with double-float
-    // samples first, their segments costing about ten times the others',
-    // so that they are handed out first and do not trail the launch) ----
+    // dispatch position: porder lists the channels of precision class 3
+    // first, their segments costing several times the others', so that they
+    // are handed out first and do not trail the launch) ----
     __shared__ int64_t s_carry2;
     __shared__ int64_t s_wsum2[32];
     // block-wide exclusive scan of one value per thread (every thread
@@ -1125,8 +1207,8 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
     }
     __syncthreads();
     int carried = 0;
-    // channels run with double-float samples: tiles of carried channels, and
-    // the class-3 channels' dispatch positions
+    // tiles of carried channels, and the dispatch positions of the channels of
+    // precision class 3
     for (int base = 0; base < C; base += blockDim.x) {
         const int c = base + tid;
         int64_t nt = 0, f3 = 0;
@@ -1171,13 +1253,14 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
         int64_t ns = 0;
         if (i < C) {
             const int c = p.porder[i];
-            const int32_t hz = __ldcg(&p.chan[c].horizon), ntl = __ldcg(&p.chan[c].ntiles);
-            if (hz >= 0) ns = ntl;
+            const int32_t hz = __ldcg(&p.chan[c].horizon), nsg = __ldcg(&p.chan[c].nseg);
+            if (hz >= 0) ns = nsg;
         }
         const int64_t q = scan(ns, s_wsum2, &s_carry2);
         if (i < C) p.tbp[i] = q;
     }
     const int64_t total2 = s_carry2;
+    __syncthreads();  // tbp complete
     const bool interleave = __syncthreads_or(carried) != 0 && C <= kMaxSortChannels;
     if (tid == 0) {
         const bool bad = __ldcg(&p.hdr->status) == SOS_ERR_WORKSPACE;
@@ -1185,6 +1268,7 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
         p.tbp[C] = total2;
         p.hdr->total_tiles = bad ? 0 : total;
         p.hdr->total_pipe = bad ? 0 : total2;
+        p.hdr->ext_segs = bad ? 0 : (n3 < C ? p.tbp[n3] : total2);
         if (!interleave) p.hdr->nrounds = 0;
     }
     if (!interleave) return;
@@ -1296,6 +1380,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(Params p) {
         h->key_kmax = p.kmax;
         h->key_C = p.C;
         h->key_seg = p.seg;
+        h->key_fair = key_fair(p);
         h->key_cap = p.cap_tiles;
         h->key_valid = 1;
         h->last_recomputed = s_changed;

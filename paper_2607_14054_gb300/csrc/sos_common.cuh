@@ -50,7 +50,8 @@ struct WsHeader {
     uint32_t plan_changed;  // channels recomputed by the running plan launch
     int64_t key_seg, key_cap;
     int32_t last_recomputed;  // channels the latest plan recomputed
-    uint32_t pad2[3];
+    int32_t key_fair;
+    int64_t ext_segs;  // of total_pipe: segments of the channels of precision class 3
 };
 static_assert(sizeof(WsHeader) == 128, "header size");
 
@@ -70,7 +71,7 @@ struct ChanInfo {
     int64_t len;      // samples
     int32_t K;        // sections used
     int32_t mode;     // 1: b0 factored out of every section (Sec. II, Eq. simple_second_order)
-    int32_t ntiles;   // tiles of this channel (dispatch)
+    int32_t ntiles;   // tiles of this channel (sos_plan_query; the look-back's dispatch)
     int32_t err;      // coefficient error found by the plan kernel (sos_status), 0 if none
     int64_t slot;     // first look-back slot of the channel (ceil(len / T) slots)
     int32_t horizon;  // >= 0: memory horizon P (segments start P samples early, no
@@ -78,8 +79,10 @@ struct ChanInfo {
     int16_t single;   // 1: the whole channel is one segment (backward plans)
     int16_t ext;      // precision class: 0 FP32; 1, 2: the largest section level
                       // (Coef32::misc.w); 3: double-float samples throughout
-    int64_t seg;      // segment length of a channel with a horizon (a multiple of 32 N,
-                      // at least 2 P)
+    int64_t seg;      // segment length of a channel with a horizon (a multiple of 16)
+    int32_t nseg;     // its segments
+    int32_t zdecay;   // samples after which the response of an arbitrary initial state has
+                      // died out (at least P)
     int32_t minseg;   // the shortest segment length the horizon allows (P, whole
                       // groups), 0 without a horizon
     int32_t minseg_z; // the same, also long enough for the response of an arbitrary
@@ -88,7 +91,7 @@ struct ChanInfo {
                          // samples, the others in FP32
     int32_t pad;
 };
-static_assert(sizeof(ChanInfo) == 72, "channel table entry");
+static_assert(sizeof(ChanInfo) == 80, "channel table entry");
 
 // A channel's memory horizon P is the shortest warm-up after which the
 // cascade's impulse-response tail, summed in absolute value, is below
@@ -109,6 +112,11 @@ constexpr double kCrKappaMax = 100.0;
 // backward call, where channels without a horizon become single segments.
 constexpr int32_t kFlagBackwardPlan = 1 << 16;
 
+// Samples per lane of a precision class 3 channel on the warp-segment and
+// streaming kernels: its double-float code needs the registers that a chunk
+// of 64 would take (the plan builds such a channel's powers for this N).
+__host__ __device__ constexpr int ext_n(int N) { return N == 64 ? 32 : N; }
+
 // Per (channel, section) FP32 coefficients and transition-matrix powers.
 // The DF2T state transition of one sample is A = [[-a1, 1], [-a2, 0]];
 // Phi = A^N advances one lane chunk, Psi = A^{N L} one warp group.  All
@@ -118,7 +126,15 @@ struct __align__(16) Coef32 {
     float4 ab;            // a1, a2, b1, b2  (b1, b2 divided by b0 when factored)
     float4 misc;          // b0, G_k (cumulative gain), 1/G_k, 1 if extended precision
     float4 braw;          // b0, b1, b2 normalised by a0 only (the adjoint's FIR)
-    float4 phi_pow[5];    // Phi^(2^j), j = 0..4 (lane scan)
+    // read together by the warp-segment kernel and the section pipeline: the
+    // powers Phi^(2^j), j = 0..4 (lane scan), A^(N/2) and A^(N/4) (the joins of a
+    // lane chunk's quarters) in the basis s1 = z1, s2 = (z2 - (a1/2) z1) / w, and w,
+    // 1/w.  With w = sqrt|a1^2/4 - a2| A is there [[c, w], [-w, c]] (complex poles)
+    // or [[c, w], [w, c]] (real ones), c = -a1/2; w is at least 1 - r, r the larger
+    // pole radius, so that coincident poles have a basis too
+    float4 phi_c[7];
+    float4 cpl;           // w, 1/w
+    float4 phi_pow[5];    // Phi^(2^j), j = 0..4 (lane scan), DF2T basis
     float4 psi_pow[4];    // Psi^(2^r), r = 0..3 (warp scan)
     float4 psi_w[16];     // Psi^w, w = 0..15 (fold the tile state into warp w)
     float4 lane_pow[32];  // Phi^l, l = 0..31 (fold the warp state into lane l)
@@ -132,10 +148,7 @@ struct __align__(16) Coef32 {
     float4 cr_tpow[5];    // C^(2^j), row-major
     float4 cr_misc;       // e_n, f_n, kappa = max |g_i|, 1 if CR is used for this section
     // read only by sections that run in extended precision (misc.w): the low
-    // parts of phi_pow and lane_pow (each power = hi + lo in double-float)
-    // and of a1, a2 (alo.x, alo.y; the exact a_i = ab + alo to 48 bits)
-    float4 phi_lo[5];
-    float4 lane_lo[32];
+    // parts of a1, a2 (alo.x, alo.y; the exact a_i = ab + alo to 48 bits)
     float4 alo;
     // read by channels run with double-float samples: the low parts of b0,
     // b1, b2 normalised by a0 (never factored; braw holds the high parts)
@@ -145,13 +158,15 @@ struct __align__(16) Coef32 {
 // Extended precision per section (Coef32::misc.w).  Level 2 when the
 // largest entry of its powers Phi^(2^j), Phi^l exceeds kDfScanEntry (poles
 // close to z = +-1 near the unit circle: the entries grow to about
-// min(l N, 1 / sin(theta)) and the FP32 products of the lane scan cancel), or
-// when rounding a1, a2 to FP32 moves its poles by more than kDfCoefSens of
-// their distance to the circle: the lane scan and fold run in double-float
-// and the in-lane recursions add the coefficients' low parts.  Level 1 when
-// that displacement exceeds kAloCoefSens only: the low parts alone (two FMAs
-// per sample and pass).  The output's relative error from rounding a1, a2
-// is about that displacement, so level 1 keeps it below 2^-18.
+// min(l N, 1 / sin(theta)), and so does what the recursions make of a
+// rounding), or when rounding a1, a2 to FP32 moves its poles by more than
+// kDfCoefSens of their distance to the circle; level 1 when that displacement
+// exceeds kAloCoefSens only.  At both levels the in-lane recursions add the
+// coefficients' low parts (two FMAs per sample and pass): the output's
+// relative error from rounding a1, a2 is about the displacement.  The states
+// are scanned in a basis in which no power's entry is large, so the scan needs
+// no more than FP32; in a double-float range a section of level 2 gets one more
+// round of refinement.
 constexpr float kDfScanEntry = 8.f;
 constexpr double kDfCoefSens = 1e-4;
 constexpr double kAloCoefSens = 0x1p-18;
@@ -252,7 +267,12 @@ struct Params {
     int32_t W;           // warps per tile
     int32_t flags_opt;   // SOS_FLAG_*
     int32_t algo;        // recursive-stage solver: 1 PH, 2 CR where well conditioned
-    int64_t seg;         // pipeline segment length (samples, a multiple of 32 N)
+    int64_t seg;         // tile length of the channels within their horizon (samples, a
+                         // multiple of 32 N): the segments of the section pipeline and
+                         // the backward
+    int64_t wseg;        // the warp-segment kernel's segment length before the channels'
+                         // horizons, and the samples per resident warp it comes from
+    int64_t fair;
     float* ck;           // backward: forward-state checkpoints [slots][kmax][2]
     const float* gy;     // backward: dL/dy [total]
     const float* gzf;    // backward: dL/dzf [C][kmax][2], or null

@@ -44,7 +44,9 @@ __device__ __forceinline__ SegGeom seg_geom(const Params& p, int64_t d) {
     g.horizon = ci.horizon;
     g.out_lo = (int64_t)g.si * ci.seg;
     g.out_hi = (ci.single || g.out_lo + ci.seg >= ci.len) ? ci.len : g.out_lo + ci.seg;
-    g.cstart = g.si == 0 ? 0 : g.out_lo - ci.horizon;
+    // outputs that the initial state's response reaches are computed from the
+    // channel's start
+    g.cstart = g.out_lo < ci.zdecay ? 0 : g.out_lo - ci.horizon;
     g.ngroups = (int)((g.out_hi - g.cstart + kGroup - 1) / kGroup);
     return g;
 }
@@ -52,7 +54,7 @@ __device__ __forceinline__ SegGeom seg_geom(const Params& p, int64_t d) {
 struct PipeShared {
     unsigned long long bar[kPipeRing][kPipeStages];  // slot ready for stage j
     unsigned long long free_[kPipeRing];             // slot free for the loader
-    float4 phi[kMaxSections][5];                     // section k's Phi^(2^j), staged by warp 1 + k
+    float4 phi[kMaxSections][8];                     // section k's phi_c and cpl, staged by warp 1 + k
     float4 cr[kMaxSections][14];                     // section k's cyclic-reduction coefficients
     uint32_t limit;                                  // bound on each hand-over wait (polls)
 };
