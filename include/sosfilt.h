@@ -320,8 +320,8 @@ sos_status sos_apply_baseline(int32_t algorithm, const float *x, int32_t n_chann
  * initial-condition matching: the plain composition (callers that want
  * scipy's odd-extension padding pad x themselves).  Arguments as in
  * sos_filter, plus tmp: device FP32 [sum len], caller-owned scratch for the
- * intermediate signal (none of x, y, tmp may overlap).  Five launches on
- * `stream` (plan, forward pass, reversal, forward pass, reversal).  No
+ * intermediate signal (none of x, y, tmp may overlap).  The plan, then two
+ * sos_apply on `stream` whose kernels write their outputs time-reversed.  No
  * counterpart in the paper: a use of the paper's filter, the cascade run
  * twice. */
 sos_status sos_filtfilt(const float *x, const double *sos, const int32_t *K, int32_t n_channels,

@@ -14,9 +14,9 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libsosfilt.so")
 SOURCES = ["warpseg_n64.cu", "warpseg_n32.cu", "warpseg_n16.cu", "warpseg.cu", "plan.cu",
            "forward.cu", "pipe.cu", "bwd.cu", "api.cu", "static_ws.cu",
-           "filtfilt.cu", "compare.cu", "host_path.cu"]
+           "compare.cu", "host_path.cu"]
 HEADERS = ["sos_common.cuh", "sos_df.cuh", "sos_f2.cuh", "sos_kernels.cuh", "sos_async.cuh",
-           "sos_pipe.cuh", "pipe_section.cuh", "warpseg.cuh"]
+           "sos_pipe.cuh", "pipe_section.cuh", "long_section.cuh", "warpseg.cuh"]
 INCLUDE = os.path.join(os.path.dirname(HERE), "include", "sosfilt.h")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",

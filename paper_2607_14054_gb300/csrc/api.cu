@@ -16,8 +16,6 @@ int warpseg_ctas_per_sm(int N, int algo);
 int warpseg_warps_per_cta();
 cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32_t maxseg,
                           int32_t foreign, cudaStream_t stream);
-cudaError_t launch_reverse(const float* src, float* dst, const Params& p, int64_t max_len,
-                           cudaStream_t stream);
 cudaError_t launch_compare(const Params& p, int algo, int64_t seg_len, int64_t max_segs,
                            cudaStream_t stream);
 }  // namespace sosf
@@ -80,8 +78,9 @@ constexpr int kPipeCtasPerSm = 2;
 // Tile length: long enough that the warm-up before each tile is a small
 // fraction of it, short enough that the tiles of the whole call keep every
 // consumer busy: each pipeline CTA (between 8 and 64 groups of 32 N), or, for
-// the warp-segment kernel, each resident warp (at least 8192 samples and at
-// most 64 groups; it cuts its own segments, Params::wseg).
+// the warp-segment kernel, each of twelve warps per SM (at least 8192 samples
+// and at most 64 groups; it cuts its own segments, Params::wseg, except those
+// of long-memory channels).
 // CTAs per SM of a warp-segment launch: the tuning's request (flag bits
 // 8..11), at most as many as fit; 0 = as many as fit.
 int warpseg_ctas(int N, int algo, int flags) {
@@ -95,8 +94,8 @@ int64_t segment_length(int64_t total_len, int N, int algo, int flags, bool warp_
     const int sms = device_sms() > 0 ? device_sms() : 148;
     int64_t units = (int64_t)sms * kPipeCtasPerSm, gmin = 8;
     if (warp_segments) {
-        const int occ = warpseg_ctas(N, algo, flags);
-        units = (int64_t)sms * (occ > 0 ? occ : 1) * warpseg_warps_per_cta();
+        const int req = (flags >> 8) & 15;
+        units = (int64_t)sms * (req > 0 && req < 3 ? req : 3) * warpseg_warps_per_cta();
         gmin = (8192 + group - 1) / group;
     }
     int64_t g = (total_len + units * group - 1) / (units * group);
@@ -197,8 +196,8 @@ sos_status setup(int32_t n_channels, int32_t kmax, const int64_t* lengths_host, 
     p->W = tu.W;
     p->flags_opt = tu.flags;
     p->algo = tu.algo;
-    p->seg = segment_length(total_len, tu.N, tu.algo, tu.flags,
-                            (tu.flags & SOS_FLAG_SECTION_PIPELINE) == 0);
+    const bool warp_segs = (tu.flags & SOS_FLAG_SECTION_PIPELINE) == 0;
+    p->seg = segment_length(total_len, warp_segs ? ext_n(tu.N) : tu.N, tu.algo, tu.flags, warp_segs);
     {
         const int64_t group = 32LL * tu.N;
         const int64_t sms = device_sms() > 0 ? device_sms() : 148;
@@ -245,7 +244,7 @@ enum ApplyParts { kPartPipe = 1, kPartCarry = 2 };
 sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
                        const int64_t* lengths_host, const float* zi, float* y, float* zf,
                        void* workspace, size_t ws_bytes, const sos_tuning* tuning, void* stream,
-                       int parts) {
+                       int parts, bool reversed = false) {
     Params p{};
     int64_t tiles = 0, total = 0;
     const sos_status s = setup(n_channels, kmax, lengths_host, workspace, ws_bytes, tuning, &p,
@@ -262,6 +261,7 @@ sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
     p.y = y;
     p.zi = zi;
     p.zf = zf;
+    p.rev = reversed ? 1 : 0;
     // the warp-segment kernel (or the section pipeline) for the channels
     // within their memory horizon, then the look-back kernel for the others
     // (which also writes the final states of empty channels and unused
@@ -445,23 +445,16 @@ sos_status sos_filtfilt(const float* x, const double* sos, const int32_t* K, int
             for (int j = i + 1; j < 3; ++j)
                 if (b[i] < b[j] + bytes && b[j] < b[i] + bytes) return SOS_ERR_ARG;
     }
-    int64_t max_len = 0;
-    for (int32_t c = 0; c < n_channels; ++c) max_len = lengths_host[c] > max_len ? lengths_host[c] : max_len;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // forward pass (zero state), reversal, forward pass of the reversed
-    // signal, reversal: y = R H R H x
+    // two forward passes from zero state, each writing its output
+    // time-reversed: y = R H R H x
     s = sos_prepare(sos, K, n_channels, kmax, lengths, lengths_host, workspace, ws_bytes, tuning,
                     stream);
     if (s != SOS_OK) return s;
-    s = sos_apply(x, n_channels, kmax, lengths_host, nullptr, tmp, nullptr, workspace, ws_bytes,
-                  tuning, stream);
+    s = apply_parts(x, n_channels, kmax, lengths_host, nullptr, tmp, nullptr, workspace, ws_bytes,
+                    tuning, stream, kPartPipe | kPartCarry, true);
     if (s != SOS_OK) return s;
-    if (launch_reverse(tmp, y, p, max_len, st) != cudaSuccess) return SOS_ERR_CUDA;
-    s = sos_apply(y, n_channels, kmax, lengths_host, nullptr, tmp, nullptr, workspace, ws_bytes,
-                  tuning, stream);
-    if (s != SOS_OK) return s;
-    if (launch_reverse(tmp, y, p, max_len, st) != cudaSuccess) return SOS_ERR_CUDA;
-    return SOS_OK;
+    return apply_parts(tmp, n_channels, kmax, lengths_host, nullptr, y, nullptr, workspace,
+                       ws_bytes, tuning, stream, kPartPipe | kPartCarry, true);
 }
 
 sos_status sos_device_status(void* workspace, void* stream) {

@@ -530,7 +530,10 @@ __global__ void __launch_bounds__((W + 1) * 32, MINB) sos_forward_kernel(Params 
         // shared -> global, all W + 1 warps (the first `skip` samples are
         // the overlap, already stored by the previous tile; skip % 16 == 0)
         float* dst = p.y + ci.off + start;
-        if (((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) && r == KT::kTile) {
+        if (p.rev) {
+            float* mir = p.y + ci.off + ci.len - 1 - start;
+            for (int j = skip + tid; j < r; j += KT::kThreads) __stcs(mir - j, buf[S::e(j)]);
+        } else if (((reinterpret_cast<uintptr_t>(dst) & 15u) == 0) && r == KT::kTile) {
             float4* d4 = reinterpret_cast<float4*>(dst);
 #pragma unroll 4
             for (int g = (skip >> 2) + tid; g < KT::kGran; g += KT::kThreads)

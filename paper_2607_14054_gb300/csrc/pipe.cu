@@ -169,17 +169,20 @@ __global__ void __launch_bounds__(2 * kPipeThreads, 1) sos_pipe_kernel(Params p)
         for (int64_t d = d0; d < total; d += dstep) {
             const SegGeom sg = seg_geom<PC::kGroup>(p, d);
             float* dst = p.y ? p.y + sg.off + sg.cstart : nullptr;
+            int64_t rev = sg.off + sg.len - 1 - sg.cstart;  // the first sample's mirror image
             // group-relative store window [a, b)
             int a = (int)(sg.out_lo - sg.cstart);
             int b = (int)(sg.out_hi - sg.cstart);
             for (int g = 0; g < sg.ngroups; ++g, dst += PC::kGroup, a -= PC::kGroup,
-                     b -= PC::kGroup) {
+                     b -= PC::kGroup, rev -= PC::kGroup) {
                 pipe_wait(p, &sh.bar[s][kMaxSections], use & 1u, lane, sh.limit);
                 const float* slot = ring + s * SL::kFloats;
                 const int lo = a > 0 ? a : 0;
                 const int hi = b < PC::kGroup ? b : PC::kGroup;
                 const bool aligned = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
                 if (!p.y) {
+                } else if (p.rev) {
+                    for (int j = lo + lane; j < hi; j += 32) __stcs(p.y + rev - j, slot[SL::elem(j)]);
                 } else if (lo == 0 && hi == PC::kGroup && aligned) {
                     float4* d4 = reinterpret_cast<float4*>(dst);
 #pragma unroll

@@ -463,9 +463,9 @@ __device__ __forceinline__ float sum_anchor(float bound) {
 // needs no compensated recursion: every chain of dependent steps is an FP32
 // one, and the long sums are independent from sample to sample and packed.
 // (Solving the recursions step by step in double-float takes about 27
-// dependent operations per sample, twice, and a double-float scan; 64 channels
-// of 2^22 samples, K = 8, half of them in double-float: 32.6 ms that way, 14.5
-// this way.)
+// dependent operations per sample, twice, and a double-float scan; 16 channels
+// of 100,003 samples, two sections: 203 us that way, 88 this way, segments
+// included.)
 // The long sums add their products one by one to an anchor far larger than
 // the sum (sum_anchor): each addition's error comes back exactly from two
 // more FMAs, and the errors are summed beside the low parts.

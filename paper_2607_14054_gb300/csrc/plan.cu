@@ -39,6 +39,17 @@ __device__ __forceinline__ float4 to_f4(const dfm2& m) {
     return make_float4(df_to_float(m.a), df_to_float(m.b), df_to_float(m.c), df_to_float(m.d));
 }
 
+// what to_f4 dropped: x - to_f4(x) per entry, the low word of the stored
+// double-float power
+__device__ __forceinline__ float df_rest(df x) {
+    const float h = df_to_float(x);
+    return (x.hi - h) + x.lo;
+}
+
+__device__ __forceinline__ float4 to_f4_lo(const dfm2& m) {
+    return make_float4(df_rest(m.a), df_rest(m.b), df_rest(m.c), df_rest(m.d));
+}
+
 // The scan's basis (Coef32::phi_c): its scale w, and a power of A in it,
 // T^-1 R T with T = [[1, 0], [a1/2, w]].
 __device__ __forceinline__ float scan_scale(double a1, double a2) {
@@ -563,12 +574,12 @@ __device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int& t
 // the channel's tile length: the call's T, or longer when the horizon
 // needs it (a tile is at least 2 P and long enough for the initial
 // state's response to decay below the bound, rounded up to whole groups of
-// G), so that long-memory channels keep a bounded warm-up instead of being
+// GT), so that long-memory channels keep a bounded warm-up instead of being
 // carried; minseg, the shortest segment the horizon allows; zdecay, the
 // samples an initial state's response takes to decay (at least P).  -1 where
 // no horizon holds.
-__device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, float la, float ilr,
-                               float zs, float lr, int64_t& seg, int32_t& minseg,
+__device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, int64_t GT, float la,
+                               float ilr, float zs, float lr, int64_t& seg, int32_t& minseg,
                                int32_t& minseg_z, int32_t& zdecay) {
     float ptail = ilr != 0.f ? (la + __logf(h2)) * ilr : 0.f;
     // the initial state's response (each pole's share counted 2K times) has
@@ -585,7 +596,7 @@ __device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, f
     const int64_t itz = (int64_t)ceilf(tz);
     const int64_t want = 2 * P > itz ? 2 * P : itz;
     seg = T;
-    if (want > seg) seg = (want + G - 1) / G * G;
+    if (want > seg) seg = (want + GT - 1) / GT * GT;
     // the shortest segments that still start their warm-up inside the
     // channel, and past an initial state's response (the streaming mode's
     // segments, where latency, not the warm-up's share, is what counts)
@@ -594,6 +605,12 @@ __device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, f
     minseg = (int32_t)((P + G - 1) / G * G > G ? (P + G - 1) / G * G : G);
     minseg_z = (int32_t)((least + G - 1) / G * G > G ? (least + G - 1) / G * G : G);
     return (int)P;
+}
+
+// Whether a channel is one of long_section.cuh's (long memory).
+__device__ __forceinline__ bool is_long(const Params& p, int horizon) {
+    return horizon > kLongHorizon && p.algo != 2 &&
+           !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE));
 }
 
 // The warp-segment kernel's segments of a channel of memory horizon P and
@@ -605,11 +622,11 @@ __device__ int horizon_combine(bool ok, float h2, int K, int64_t T, int64_t G, f
 //    each take 8 us, one warp of four 11);
 //  - double-float sections cost several times the FP32 ones: a quarter of it;
 //  - where 2 P is longer, S grows towards 2 P (a warm-up of half the outputs)
-//    as long as S + P stays below a few times the samples per warp, so that
-//    the channels with the longest memory do not end long after the others
-//    (64 channels of 2^22 samples, P = 43K..270K: 14.5 ms against 15.1
-//    with 2 P; 16 channels of 100,003, P = 4416: 88 us against 155), but not
-//    below P/4.
+//    as long as S + P stays below twice the samples per warp (three times for
+//    double-float), so that the channels with the longest memory do not end
+//    long after the others, but not below P/4 (16 channels of 100,003, P =
+//    4416: 88 us against 155 with 2 P; 1024 clips of up to 8,200: 94 us at
+//    three times, 103 at two).
 // S + P is then rounded up to whole groups: the last one is computed anyway.
 __device__ __forceinline__ void warp_segments(const Params& p, int c, int64_t len, int64_t P,
                                               int e) {
@@ -881,7 +898,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         int64_t seg = p.seg;
         int32_t minseg = 0, minseg_z = 0, zdecay = 0;
         int P = carry_only ? -1
-                           : horizon_combine(ok, h2, Kc, p.seg, 32LL * p.N, la, ilr, zs, lr, seg,
+                           : horizon_combine(ok, h2, Kc, p.seg, 32LL * p.N, 32LL * ext_n(p.N), la, ilr, zs, lr, seg,
                                              minseg, minseg_z, zdecay);
         // a channel without a partial-fraction horizon (repeated poles)
         // takes the cruder bound: always in backward plans, which have no
@@ -899,7 +916,8 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
                 const int64_t G = 32LL * p.N;
                 P = Pf;
                 seg = p.seg;
-                if (want > seg) seg = (want + G - 1) / G * G;
+                const int64_t GT = 32LL * ext_n(p.N);
+                if (want > seg) seg = (want + GT - 1) / GT * GT;
                 zdecay = tzf > Pf ? tzf : Pf;
                 minseg = (int32_t)((Pf + G - 1) / G * G > G ? (Pf + G - 1) / G * G : G);
                 minseg_z = (int32_t)((tzf + G - 1) / G * G > minseg ? (tzf + G - 1) / G * G
@@ -927,6 +945,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
             p.chan[c].seg = P >= 0 ? seg : p.seg;
             p.chan[c].nseg = (int32_t)nt;
             p.chan[c].zdecay = zdecay;
+            p.chan[c].longm = P >= 0 && Kc > 0 && is_long(p, P) ? 1 : 0;
             if (P >= 0 && Kc == 0 && !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE)))
                 warp_segments(p, c, len, P, 0);  // (else by the first section warp)
             p.chan[c].minseg = P >= 0 ? minseg : 0;
@@ -1052,7 +1071,8 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         out32->ab = make_float4((float)a1, (float)a2, (float)(b1 * sb), (float)(b2 * sb));
         out32->alo = make_float4((float)(a1 - (double)(float)a1), (float)(a2 - (double)(float)a2),
                                  0.0f, 0.0f);
-        out32->misc = make_float4((float)b0, (float)s_G[k], s_Ginv[k], ext);
+        const bool twice = m > kRefineEntry || sens > kRefineSens;
+        out32->misc = make_float4((float)b0, (float)s_G[k], s_Ginv[k], twice ? 3.f : ext);
         out32->braw = make_float4((float)b0, (float)b1, (float)b2, 0.0f);
         out32->blo = make_float4((float)(b0 - (double)(float)b0), (float)(b1 - (double)(float)b1),
                                  (float)(b2 - (double)(float)b2), 0.0f);
@@ -1097,19 +1117,34 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         s_ext = e;
         if (s_horizon >= 0 &&
             !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE)))
-            warp_segments(p, c, p.lengths[c], s_horizon, e);
+            if (!is_long(p, s_horizon)) warp_segments(p, c, p.lengths[c], s_horizon, e);
     }
     if (s_horizon >= 0) {
+        // the powers for ext_n(N) samples per lane, the j-th squaring from there
+        auto pow2 = [&](int j) {
+            return ext_n(N) == N ? s_chain[k][j] : j == 0 ? s_part[k][0] : s_chain[k][j - 1];
+        };
+        if (is_long(p, s_horizon)) {
+            // a long-memory channel: the DF2T powers with their low parts
+            dfm2 P = dfm_identity();
+            for (int j = 0; j < 5; ++j)
+                if ((lane >> j) & 1) P = dfm_mul(P, pow2(j));
+            out32->lane_pow[lane] = to_f4(P);
+            LongCoef* far = reinterpret_cast<LongCoef*>(outdf);
+            far->lane_lo[lane] = to_f4_lo(P);
+            if (lane < 5) {
+                out32->phi_pow[lane] = to_f4(pow2(lane));
+                far->phi_lo[lane] = to_f4_lo(pow2(lane));
+            }
+        }
         if (ext_n(N) != N &&
             !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE))) {
             // a channel of precision class 3 runs with ext_n(N) = N/2 samples
             // per lane: its powers again, one squaring earlier
             asm volatile("bar.sync 4, %0;" ::"r"(32 * Kc) : "memory");
             if (s_ext >= 3 && lane < 7)
-                out32->phi_c[lane] = scan_basis(lane == 0   ? s_part[k][0]
-                                                : lane < 5 ? s_chain[k][lane - 1]
-                                                           : s_part[k][lane - 4],
-                                                a1, scan_scale(a1, a2));
+                out32->phi_c[lane] = scan_basis(lane < 5 ? pow2(lane) : s_part[k][lane - 4], a1,
+                                                scan_scale(a1, a2));
         }
         return true;
     }
@@ -1178,8 +1213,8 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
     __shared__ int64_t s_wsum[32];
     // ---- prefixes: look-back tiles of the carried channels (tb, by
     // channel) and segments of the channels within their horizon (tbp, by
-    // dispatch position: porder lists the channels of precision class 3
-    // first, their segments costing several times the others', so that they
+    // dispatch position: porder lists the long-memory channels first, and
+    // before the others of each kind the channels of precision class 3, their segments costing several times the others', so that they
     // are handed out first and do not trail the launch) ----
     __shared__ int64_t s_carry2;
     __shared__ int64_t s_wsum2[32];
@@ -1206,44 +1241,46 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
         s_carry2 = 0;
     }
     __syncthreads();
-    int carried = 0;
-    // tiles of carried channels, and the dispatch positions of the channels of
-    // precision class 3
+    int carried = 0, widest = 0;
+    // tiles of carried channels; the most sections of a long-memory channel
     for (int base = 0; base < C; base += blockDim.x) {
         const int c = base + tid;
-        int64_t nt = 0, f3 = 0;
+        int64_t nt = 0;
         if (c < C) {
             // written by other blocks of this launch: read past L1
             const int32_t hz = __ldcg(&p.chan[c].horizon), ntl = __ldcg(&p.chan[c].ntiles);
-            const int16_t ext = __ldcg(&p.chan[c].ext);
             if (hz < 0) {
                 nt = ntl;
                 if (nt > 1) carried = 1;
-            } else {
-                f3 = ext >= 3 ? 1 : 0;
+            } else if (__ldcg(&p.chan[c].longm)) {
+                const int K = __ldcg(&p.chan[c].K);
+                widest = widest > K ? widest : K;
             }
         }
         const int64_t t0 = scan(nt, s_wsum, &s_carry);
-        const int64_t q0 = scan(f3, s_wsum2, &s_carry2);
-        if (c < C) {
-            p.tb[c] = t0;
-            if (f3) p.porder[q0] = c;
-        }
+        if (c < C) p.tb[c] = t0;
     }
-    const int64_t total = s_carry, n3 = s_carry2;
-    __syncthreads();
-    if (tid == 0) s_carry2 = 0;
-    __syncthreads();
-    for (int base = 0; base < C; base += blockDim.x) {
-        const int c = base + tid;
-        int64_t f = 0;
-        if (c < C) {
-            const int32_t hz = __ldcg(&p.chan[c].horizon);
-            const int16_t ext = __ldcg(&p.chan[c].ext);
-            f = (hz >= 0 && ext >= 3) ? 0 : 1;
+    const int64_t total = s_carry;
+    const int team = __syncthreads_or(widest > 4) ? 4 : __syncthreads_or(widest > 2) ? 2 : 1;
+    // dispatch positions: long-memory channels (double-float ones first), then
+    // the others (the same), as categories 0..3
+    int64_t first_of[4];
+    for (int cat = 0; cat < 4; ++cat) {
+        first_of[cat] = s_carry2;
+        __syncthreads();
+        for (int base = 0; base < C; base += blockDim.x) {
+            const int c = base + tid;
+            int64_t f = 0;
+            if (c < C) {
+                const bool far = __ldcg(&p.chan[c].longm) != 0;
+                const bool df3 =
+                    __ldcg(&p.chan[c].horizon) >= 0 && __ldcg(&p.chan[c].ext) >= 3;
+                f = (far ? 0 : 2) + (df3 ? 0 : 1) == cat ? 1 : 0;
+            }
+            const int64_t q = scan(f, s_wsum2, &s_carry2);
+            if (c < C && f) p.porder[q] = c;
         }
-        const int64_t q = scan(f, s_wsum2, &s_carry2);
-        if (c < C && f) p.porder[n3 + q] = c;
+        __syncthreads();
     }
     __syncthreads();  // porder complete (block-wide visibility of its global writes)
     if (tid == 0) s_carry2 = 0;
@@ -1268,7 +1305,9 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
         p.tbp[C] = total2;
         p.hdr->total_tiles = bad ? 0 : total;
         p.hdr->total_pipe = bad ? 0 : total2;
-        p.hdr->ext_segs = bad ? 0 : (n3 < C ? p.tbp[n3] : total2);
+        p.hdr->long_segs = bad ? 0 : (first_of[2] < C ? p.tbp[first_of[2]] : total2);
+        p.hdr->ext_segs = bad ? 0 : (first_of[3] < C ? p.tbp[first_of[3]] : total2);
+        p.hdr->long_team = team;
         if (!interleave) p.hdr->nrounds = 0;
     }
     if (!interleave) return;

@@ -51,9 +51,14 @@ struct WsHeader {
     int64_t key_seg, key_cap;
     int32_t last_recomputed;  // channels the latest plan recomputed
     int32_t key_fair;
-    int64_t ext_segs;  // of total_pipe: segments of the channels of precision class 3
+    // the segments are listed with those of the long-memory channels first, then
+    // those of precision class 3: where each of the two ends
+    int64_t ext_segs, long_segs;
+    unsigned long long long_next;  // long-memory segments handed out to the teams
+    uint32_t long_done;            // teams of the running launch that have finished them
+    int32_t long_team;             // warps per team: 1, 2 or 4
 };
-static_assert(sizeof(WsHeader) == 128, "header size");
+static_assert(sizeof(WsHeader) == 152, "header size");
 
 // Per-channel record of the plan cache: the raw sos rows (bit patterns), K
 // and length from which the channel's tables were last built.
@@ -89,7 +94,7 @@ struct ChanInfo {
                       // initial state to die out
     int16_t dflo, dfhi;  // precision class 3: sections dflo..dfhi run with double-float
                          // samples, the others in FP32
-    int32_t pad;
+    int32_t longm;    // 1: a long-memory channel (kLongHorizon) of a warp-segment plan
 };
 static_assert(sizeof(ChanInfo) == 80, "channel table entry");
 
@@ -102,6 +107,13 @@ static_assert(sizeof(ChanInfo) == 80, "channel table entry");
 // far below FP32 rounding.  Longer memories (P > T / 2, poles on or near the
 // unit circle, coincident poles) keep the decoupled look-back.
 constexpr float kHorizonEps = 0x1p-30f;
+
+// Channels with a longer horizon keep the scalar order of operations of
+// long_section.cuh on the warp-segment kernel (there the reason), in segments
+// of their tile length.  The line: poles at radius 0.995 have horizons of about
+// 5,300 samples and rounding errors below 1e-5 either way; at 0.999 the horizon
+// is above 20,000 and the errors reach 1e-3, in either order, but other ones.
+constexpr int kLongHorizon = 8192;
 
 // Cyclic reduction divides by e_i at every level (c_i = e_i - f_i / e_i);
 // a section whose |f_i / e_i| exceeds this at some level keeps PH, which
@@ -124,7 +136,7 @@ __host__ __device__ constexpr int ext_n(int N) { return N == 64 ? 32 : N; }
 // stored row-major in a float4 (m00, m01, m10, m11).
 struct __align__(16) Coef32 {
     float4 ab;            // a1, a2, b1, b2  (b1, b2 divided by b0 when factored)
-    float4 misc;          // b0, G_k (cumulative gain), 1/G_k, 1 if extended precision
+    float4 misc;          // b0, G_k (cumulative gain), 1/G_k, precision level
     float4 braw;          // b0, b1, b2 normalised by a0 only (the adjoint's FIR)
     // read together by the warp-segment kernel and the section pipeline: the
     // powers Phi^(2^j), j = 0..4 (lane scan), A^(N/2) and A^(N/4) (the joins of a
@@ -165,10 +177,16 @@ struct __align__(16) Coef32 {
 // coefficients' low parts (two FMAs per sample and pass): the output's
 // relative error from rounding a1, a2 is about the displacement.  The states
 // are scanned in a basis in which no power's entry is large, so the scan needs
-// no more than FP32; in a double-float range a section of level 2 gets one more
-// round of refinement.
+// no more than FP32.  misc.w is 3 for the few sections of level 2 whose FP32
+// solve may be off by more than about 1e-4 (poles within about 1/64 of z = +-1):
+// in a double-float range they get a second round of refinement (measured with
+// the refined solve on channels of radius 0.999..0.9999 too: one round
+// everywhere left one of 64 channels at 1.1e-2 instead of 4e-4 and changed no
+// other; two rounds at all of level 2 took 14.5 instead of 11.9 ms).
 constexpr float kDfScanEntry = 8.f;
 constexpr double kDfCoefSens = 1e-4;
+constexpr float kRefineEntry = 64.f;
+constexpr float kRefineSens = 1e-3f;
 constexpr double kAloCoefSens = 0x1p-18;
 
 // A channel is run with double-float samples throughout (ChanInfo::ext = 3)
@@ -199,6 +217,14 @@ struct __align__(16) CoefDF {
     float4 theta_pow[33][2];
     float4 theta_hi[18][2];
 };
+
+// In its place for long-memory channels, which are never carried by the
+// look-back: the low parts of phi_pow and lane_pow.
+struct __align__(16) LongCoef {
+    float4 phi_lo[5];
+    float4 lane_lo[32];
+};
+static_assert(sizeof(LongCoef) <= sizeof(CoefDF), "LongCoef lies in CoefDF's place");
 
 // Look-back words, per (section, tile): the tile's inclusive (true outgoing)
 // state as four 64-bit words (z1.hi, z1.lo, z2.hi, z2.lo) and its aggregate
@@ -280,6 +306,7 @@ struct Params {
     float* gzi;          // backward: dL/dzi [C][kmax][2], or null
     double* gacc;        // backward: [C][kmax][5] sums for b0, b1, b2, a1, a2
     int64_t total;       // samples of all channels
+    int64_t rev;         // 1: each channel's output is written time-reversed (sos_filtfilt)
 };
 
 // Launch of fn(p); early: programmatic dependent launch, the kernel may be

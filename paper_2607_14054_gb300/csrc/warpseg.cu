@@ -17,7 +17,12 @@ namespace {
 const void* ws_fn(int N, bool cr) {
     return N == 16 ? warpseg_fn_16(cr) : N == 32 ? warpseg_fn_32(cr) : warpseg_fn_64(cr);
 }
-size_t ws_smem(int N) { return sizeof(float) * 32 * (size_t)(N + 4) * 2 * kWsWarps; }
+// two group slots per warp, or twelve slots for ext_n(N) (WsCfg::kSmem)
+size_t ws_smem(int N) {
+    const size_t own = 32 * (size_t)(N + 4) * 2 * kWsWarps;
+    const size_t far = 32 * (size_t)(ext_n(N) + 4) * 12;
+    return sizeof(float) * (own > far ? own : far);
+}
 }  // namespace
 
 // CTAs of the warp-segment kernel (algo 2: the cyclic-reduction one)

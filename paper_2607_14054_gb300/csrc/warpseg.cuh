@@ -18,7 +18,7 @@
 
 #include <type_traits>
 
-#include "pipe_section.cuh"
+#include "long_section.cuh"
 #include "sos_pipe.cuh"
 
 namespace sosf {
@@ -43,7 +43,11 @@ struct WsCfg {
     static constexpr int kGroup = 32 * N;
     static constexpr int kGran = kGroup / 4;
     static constexpr int kSlot = 32 * (N + 4);  // floats per slot
-    static constexpr size_t kSmem = sizeof(float) * kSlot * 2 * kWsWarps;
+    // two slots per warp; the long-memory teams share twelve for ext_n(N)
+    static constexpr int kLongSlot = 32 * (ext_n(N) + 4);
+    static constexpr int kFloats =
+        kSlot * 2 * kWsWarps > 12 * kLongSlot ? kSlot * 2 * kWsWarps : 12 * kLongSlot;
+    static constexpr size_t kSmem = sizeof(float) * kFloats;
 };
 
 // the asynchronous copies of one group (rem samples left in the channel)
@@ -69,6 +73,7 @@ __device__ __forceinline__ void ws_load(const float* src, int64_t rem, float* sl
 // through the section loop (at N = 64 the chunk alone takes 64 of the 168).
 struct WsSeg {
     int64_t base;   // packed index of the first computed sample (off + cstart)
+    int64_t rbase;  // packed index of that sample's mirror image in the channel
     int64_t nbase;  // of the warp's next segment's, -1 if there is none to prefetch
     int rem, nrem;  // samples of the channel from there on (capped)
     int a, b;       // the segment's own outputs, relative to base
@@ -100,6 +105,7 @@ struct WsShared {
     WsCoef cf[kWsWarps][kMaxSections];
     WsSeg seg[kWsWarps];
     Params p;                             // the call's parameters
+    int64_t item[kWsWarps];               // the segment a long-memory team works on
 };
 static __shared__ WsShared s_ws;
 extern __shared__ float4 s_ws_slots[];
@@ -143,8 +149,8 @@ __device__ __forceinline__ void ws_stage(const Coef32* cf0, int K, WsCoef* sc, i
 
 // Sections [k0, k1) of a channel run with double-float samples over one
 // group (kPrecDF): on entry the lane's row holds its chunk of the range's
-// FP32 input, on exit the chunk of its output, rounded once.  Sections whose powers or poles are
-// ill-conditioned (level 2) get a second round of refinement.
+// FP32 input, on exit the chunk of its output, rounded once.  The most
+// ill-conditioned sections get a second round of refinement.
 template <int N, bool ZF>
 __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int owner, int mq) {
     const Params& p = s_ws.p;
@@ -169,7 +175,7 @@ __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int
         df z1{zz.x, zz.y}, z2{zz.z, zz.w};
         pipe_section_dfx<N, ZF>(xh, xl, mx, sd, sc[k].phi,
                                 make_float2(sc[k].cpl.x, sc[k].cpl.y),
-                                sc[k].misc.w > 1.5f ? 2 : 1, z1, z2, lane == owner, mq, row,
+                                sc[k].misc.w > 2.5f ? 2 : 1, z1, z2, lane == owner, mq, row,
                                 zf_dst);
         if (lane == 0) zs[k] = make_float4(z1.hi, z1.lo, z2.hi, z2.lo);
     }
@@ -287,6 +293,46 @@ __device__ __forceinline__ void ws_filter(int row_at, int c, int K, int owner, i
     }
 }
 
+// Coalesced stores of samples [lo, hi) of the group in `slot`, whose first
+// sample is number `at` of the packed output and whose mirror image (p.rev:
+// the zero-phase filter's passes write time-reversed, where a pass for the
+// reversal took 27 us for 64 channels of 100,003 beside a filtering kernel of
+// 32) is number `rat`.
+template <int N>
+__device__ __forceinline__ void ws_store(const Params& p, const float* slot, int lane, int lo,
+                                         int hi, int64_t at, int64_t rat) {
+    using SL = SlotLayout<N>;
+    using WC = WsCfg<N>;
+    if (p.rev) {
+        float* dst = p.y + rat;  // sample j goes to dst[-j]
+        if (((lo | hi) & 3) == 0 && (reinterpret_cast<uintptr_t>(dst - 3) & 15u) == 0) {
+            for (int i = (lo >> 2) + lane; i < (hi >> 2); i += 32) {
+                const float4 t = *reinterpret_cast<const float4*>(slot + SL::gran(i));
+                __stcs(reinterpret_cast<float4*>(dst - 4 * i - 3), make_float4(t.w, t.z, t.y, t.x));
+            }
+        } else {
+            for (int j = lo + lane; j < hi; j += 32) __stcs(dst - j, slot[SL::elem(j)]);
+        }
+    } else {
+        float* dst = p.y + at;
+        const bool aligned = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
+        if (lo == 0 && hi == WC::kGroup && aligned) {
+            float4* d4 = reinterpret_cast<float4*>(dst);
+#pragma unroll
+            for (int i = 0; i < WC::kGran / 32; ++i)
+                __stcs(d4 + i * 32 + lane,
+                       *reinterpret_cast<const float4*>(slot + SL::gran(i * 32 + lane)));
+        } else if (((lo | hi) & 3) == 0 && aligned) {
+            float4* d4 = reinterpret_cast<float4*>(dst);
+            for (int i = (lo >> 2) + lane; i < (hi >> 2); i += 32)
+                __stcs(d4 + i, *reinterpret_cast<const float4*>(slot + SL::gran(i)));
+        } else {
+            for (int j = lo + lane; j < hi; j += 32) __stcs(dst + j, slot[SL::elem(j)]);
+        }
+    }
+    __syncwarp();
+}
+
 // Group g of a segment: prefetch the next group, filter this one (ws_filter),
 // store the segment's own outputs.  base: the warp's two group slots, `cur`
 // holding this group.
@@ -313,25 +359,9 @@ __device__ __forceinline__ void ws_group(const Params& p, const volatile WsSeg& 
     ws_filter<N, FACT, CR, ZF, PREC>(base + cur * WC::kSlot + lane * SL::kRow, sg.c, sg.K,
                                      ZF ? (sg.zrel % WC::kGroup) / N : 0, ZF ? sg.zrel % N : 0);
     __syncwarp();
-    // coalesced stores of the segment's own samples of this group
     const int a = sg.a - g * WC::kGroup, b = sg.b - g * WC::kGroup;
-    const int lo = a > 0 ? a : 0, hi = b < WC::kGroup ? b : WC::kGroup;
-    float* dst = p.y + sg.base + (int64_t)g * WC::kGroup;
-    const bool aligned = (reinterpret_cast<uintptr_t>(dst) & 15u) == 0;
-    if (lo == 0 && hi == WC::kGroup && aligned) {
-        float4* d4 = reinterpret_cast<float4*>(dst);
-#pragma unroll
-        for (int i = 0; i < WC::kGran / 32; ++i)
-            __stcs(d4 + i * 32 + lane,
-                   *reinterpret_cast<const float4*>(slot + SL::gran(i * 32 + lane)));
-    } else if (((lo | hi) & 3) == 0 && aligned) {
-        float4* d4 = reinterpret_cast<float4*>(dst);
-        for (int i = (lo >> 2) + lane; i < (hi >> 2); i += 32)
-            __stcs(d4 + i, *reinterpret_cast<const float4*>(slot + SL::gran(i)));
-    } else {
-        for (int j = lo + lane; j < hi; j += 32) __stcs(dst + j, slot[SL::elem(j)]);
-    }
-    __syncwarp();
+    ws_store<N>(p, slot, lane, a > 0 ? a : 0, b < WC::kGroup ? b : WC::kGroup,
+                sg.base + (int64_t)g * WC::kGroup, sg.rbase - (int64_t)g * WC::kGroup);
 }
 
 // All groups of one segment through all K sections (one warp).  On return
@@ -390,6 +420,7 @@ __device__ __forceinline__ void ws_set(const Params& p, volatile WsSeg& ws, cons
                                        int lane) {
     if (lane == 0) {
         ws.base = sg.off + sg.cstart;
+        ws.rbase = sg.off + sg.len - 1 - sg.cstart;
         ws.rem = ws_cap(sg.len - sg.cstart);
         ws.a = (int)(sg.out_lo - sg.cstart);
         ws.b = (int)(sg.out_hi - sg.cstart);
@@ -413,8 +444,8 @@ __device__ __forceinline__ void ws_run_segment(const Params& p, int base, int la
     if (K == 0) {
         // identity channel: copy the segment's own samples (nothing of it is
         // in the slots, but the next segment's first group is due)
-        for (int64_t i = sg.base + sg.a + lane; i < sg.base + sg.b; i += 32)
-            p.y[i] = __ldg(p.x + i);
+        for (int i = sg.a + lane; i < sg.b; i += 32)
+            p.y[p.rev ? sg.rbase - i : sg.base + i] = __ldg(p.x + sg.base + i);
         const int nxt = sg.cur ^ 1;
         __syncwarp();
         if (sg.nbase >= 0)
@@ -441,6 +472,212 @@ __device__ __forceinline__ void ws_run_segment(const Params& p, int base, int la
         if (fact) ws_segment<N, true, false, kPrecF32>(p, sg, base, lane);
         else ws_segment<N, false, false, kPrecF32>(p, sg, base, lane);
     }
+}
+
+// ---- long-memory channels (long_section.cuh) ----
+
+__device__ __forceinline__ void team_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// Sections [k0, k1) of a long-memory channel over the group in `hi` (and, in
+// the double-float range, `lo`: the low parts), lane rows of N samples; the
+// last stage multiplies the split-off gain in.  ZF: the group holds the
+// channel's last sample (element mq of lane owner's chunk).
+template <int N, bool ZF>
+__device__ __forceinline__ void long_stage(const Params& p, const ChanInfo& ci, int c, int k0,
+                                           int k1, bool last, float* hi, float* lo, float4* zs,
+                                           int lane, int owner, int mq) {
+    constexpr int R = SlotLayout<N>::kRow;
+    const Coef32* cf0 = p.c32 + (int64_t)c * p.kmax;
+    float* row = hi + lane * R;
+    float* lrow = lo + lane * R;
+    const bool df3 = ci.ext >= 3, fact = !df3 && ci.mode != 0;
+    const int dlo = df3 ? ci.dflo : 8, dhi = df3 ? ci.dfhi : -1;
+    float v[N];
+    row_to_chunk<N>(v, row);
+#pragma unroll 1
+    for (int k = k0; k < k1; ++k) {
+        const Coef32* cf = cf0 + k;
+        const LongCoef* lc =
+            reinterpret_cast<const LongCoef*>(p.cdf + (int64_t)c * p.kmax + k);
+        float* zf_dst = ZF ? p.zf + ((int64_t)c * p.kmax + k) * 2 : nullptr;
+        const float4 zz = zs[k];
+        const float4 lp = cf->lane_pow[lane];
+        float4 zo;
+        if (k >= dlo && k <= dhi) {
+            if (k == dlo) {
+                // the range's input is FP32: its low parts start at zero
+#pragma unroll
+                for (int b = 0; b < N / 4; ++b)
+                    reinterpret_cast<float4*>(lrow)[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            df z1{zz.x, zz.y}, z2{zz.z, zz.w};
+            long_section_dfx<N, ZF>(v, lrow, load_secdf(cf), cf->phi_pow, lc->phi_lo, lp,
+                                    lc->lane_lo[lane], z1, z2, lane == owner, mq, zf_dst);
+            zo = make_float4(z1.hi, z1.lo, z2.hi, z2.lo);
+            if (k == dhi) {
+                // the range's output, rounded once
+#pragma unroll
+                for (int b = 0; b < N / 4; ++b) {
+                    const float4 l = reinterpret_cast<const float4*>(lrow)[b];
+                    v[4 * b + 0] += l.x;
+                    v[4 * b + 1] += l.y;
+                    v[4 * b + 2] += l.z;
+                    v[4 * b + 3] += l.w;
+                }
+            }
+        } else {
+            float4 ab = cf->ab;
+            float b0 = fact ? 1.f : cf->misc.x;
+            if (df3) {
+                const float4 br = cf->braw;
+                ab.z = br.y;
+                ab.w = br.z;
+                b0 = br.x;
+            }
+            const float G = ZF && fact ? cf->misc.y : 1.f, lvl = cf->misc.w;
+            const float4 al = cf->alo;
+            const float2 alo = make_float2(al.x, al.y);
+            const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+            float z1 = zz.x, z2 = zz.z;
+            if (lvl > 1.5f)
+                long_section<N, ZF, true, true>(v, ab, b0, cf->phi_pow, lp, z1, z2, lane == owner,
+                                                mq, row, zf_dst, G, alo, lc->phi_lo,
+                                                lc->lane_lo[lane]);
+            else if (lvl > 0.5f)
+                long_section<N, ZF, true, false>(v, ab, b0, cf->phi_pow, lp, z1, z2, lane == owner,
+                                                 mq, row, zf_dst, G, alo, nullptr, none);
+            else
+                long_section<N, ZF, false, false>(v, ab, b0, cf->phi_pow, lp, z1, z2,
+                                                  lane == owner, mq, row, zf_dst, G, alo, nullptr,
+                                                  none);
+            zo = make_float4(z1, 0.f, z2, 0.f);
+        }
+        __syncwarp();
+        if (lane == 0) zs[k] = zo;
+    }
+    if (last && fact) {
+        const float Gk = cf0[ci.K - 1].misc.y;
+#pragma unroll
+        for (int m = 0; m < N; ++m) v[m] *= Gk;
+    }
+    chunk_to_row<N>(v, row);
+    __syncwarp();
+}
+
+// The segments of the long-memory channels.  A segment is a sequential walk of
+// up to a thousand groups, most of it latency of dependent steps, and such a
+// channel has few segments, so a team of q warps (q = 1, 2 or 4 for up to 2, 4
+// and 8 sections) shares one: stage w of the team runs its share of the
+// sections on group s - w while the stages before it run theirs on the groups
+// after it, one team barrier per step; every section sees the same groups in
+// the same order as if one warp ran them all (64 channels of 2^22 samples, K =
+// 8: 20.7 ms, 34.2 with a warp per segment; 9 channels of 300,007, K = 3, the
+// same digits).  The shares are cut by cost (double-float 6, double-float scan 2).
+// N: samples per lane.
+template <int N>
+__device__ __forceinline__ void ws_long_phase(const Params& p, int lane) {
+    constexpr int G = 32 * N, kSlot = 32 * SlotLayout<N>::kRow;
+    const int64_t total = p.hdr->long_segs;
+    if (total <= 0) return;
+    const int q = p.hdr->long_team;
+    const int w = ws_warp(), team = w / q, stage = w % q;
+    // the team's 3 q slots: groups in flight, then their low parts
+    const int nh = q == 1 ? 2 : q == 2 ? 3 : 6, nl = 3 * q - nh;
+    float* slots = ws_slots(team * 3 * q * kSlot);
+    float4* zs = s_ws.z[team];
+    const int bar = 1 + team, threads = 32 * q;
+    for (;;) {
+        if (stage == 0 && lane == 0)
+            s_ws.item[team] = (int64_t)atomicAdd(&p.hdr->long_next, 1ull);
+        team_sync(bar, threads);
+        const int64_t item = s_ws.item[team];
+        if (item >= total) break;
+        const SegGeom sg = seg_geom<G>(p, item);
+        const ChanInfo ci = p.chan[sg.c];
+        const int K = sg.K, ng = sg.ngroups;
+        const Coef32* cf0 = p.c32 + (int64_t)sg.c * p.kmax;
+        // this stage's sections
+        int k0 = 0, k1 = 0;
+        {
+            auto cost = [&](int k) {
+                return ci.ext >= 3 && k >= ci.dflo && k <= ci.dfhi ? 6
+                                                                   : (cf0[k].misc.w > 1.5f ? 2 : 1);
+            };
+            int sum = 0, acc = 0;
+            for (int k = 0; k < K; ++k) sum += cost(k);
+            for (int k = 0; k < K; ++k) {
+                // section k goes to the stage its middle falls into
+                const int ck = cost(k), st = (2 * acc + ck) * q / (2 * sum);
+                acc += ck;
+                if (st < stage) k0 = k + 1;
+                if (st <= stage) k1 = k + 1;
+            }
+        }
+        const float* src = p.x + sg.off + sg.cstart;
+        const int rem = ws_cap(sg.len - sg.cstart);
+        const int zrel =
+            p.zf && sg.out_hi == sg.len ? (int)(sg.len - 1 - sg.cstart) : -1;
+        if (stage == 0) {
+            if (lane < K) {
+                float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (sg.cstart == 0 && p.zi) {
+                    const float gi = ci.mode != 0 && ci.ext < 3 ? cf0[lane].misc.z : 1.f;
+                    z.x = p.zi[((int64_t)sg.c * p.kmax + lane) * 2 + 0] * gi;
+                    z.z = p.zi[((int64_t)sg.c * p.kmax + lane) * 2 + 1] * gi;
+                }
+                zs[lane] = z;
+            }
+            ws_load<N>(src, rem, slots, lane);
+        }
+        team_sync(bar, threads);
+#pragma unroll 1
+        for (int s = 0; s < ng + q - 1; ++s) {
+            const int g = s - stage;
+            if (stage == 0 && s < ng) {
+                if (s + 1 < ng) {
+                    ws_load<N>(src + (int64_t)(s + 1) * G, rem - (s + 1) * G,
+                               slots + (s + 1) % nh * kSlot, lane);
+                    cp_async_wait1();
+                } else {
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                }
+                __syncwarp();
+            }
+            if (g >= 0 && g < ng) {
+                float* hi = slots + g % nh * kSlot;
+                float* lo = slots + (nh + g % nl) * kSlot;
+                const bool last = stage == q - 1;
+                if (k0 < k1 || last) {
+                    if (zrel >= 0 && g == ng - 1)
+                        long_stage<N, true>(p, ci, sg.c, k0, k1, last, hi, lo, zs, lane,
+                                            zrel % G / N, zrel % N);
+                    else
+                        long_stage<N, false>(p, ci, sg.c, k0, k1, last, hi, lo, zs, lane, 0, 0);
+                }
+                if (last) {
+                    const int64_t at = sg.off + sg.cstart + (int64_t)g * G;
+                    const int64_t a = sg.out_lo - sg.cstart - (int64_t)g * G;
+                    const int64_t b = sg.out_hi - sg.cstart - (int64_t)g * G;
+                    ws_store<N>(p, hi, lane, (int)(a > 0 ? a : 0), (int)(b < G ? b : G), at,
+                                2 * sg.off + sg.len - 1 - at);
+                }
+            }
+            team_sync(bar, threads);
+        }
+    }
+    // the last team to finish resets the hand-out for the next launch
+    if (stage == 0 && lane == 0) {
+        __threadfence();
+        const unsigned prev = atomicAdd(&p.hdr->long_done, 1u);
+        if (prev + 1 == gridDim.x * (kWsWarps / q)) {
+            p.hdr->long_next = 0;
+            p.hdr->long_done = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();  // the slots go to the warps again
 }
 
 // The call's parameters to shared memory (whole CTA).
@@ -470,7 +707,9 @@ __global__ void __launch_bounds__(kWsThreads, ws_ctas_per_sm<N>())
     const int base = ws_slot_base<N>();
     float* slots = ws_slots(base);
     volatile WsSeg& ws = s_ws.seg[w];
-    const int64_t total = p.hdr->total_pipe;  // segments of the latest plan
+    ws_long_phase<ext_n(N)>(p, lane);
+    const int64_t skip = p.hdr->long_segs;
+    const int64_t total = p.hdr->total_pipe - skip;  // the other segments of the latest plan
     // segments: the first gridDim.x kWsWarps one per warp, the rest handed out
     // in order as warps come free (segments differ in length across uneven
     // channels).  The first round goes across the CTAs, and so the SMs, before
@@ -491,8 +730,8 @@ __global__ void __launch_bounds__(kWsThreads, ws_ctas_per_sm<N>())
     // ---- the segments of precision class 3, which come first ----
     constexpr int NX = ext_n(N);
 #pragma unroll 1
-    while (d < p.hdr->ext_segs) {
-        const SegGeom sg = seg_geom<WsCfg<NX>::kGroup>(p, d);
+    while (d < p.hdr->ext_segs - skip) {
+        const SegGeom sg = seg_geom<WsCfg<NX>::kGroup>(p, skip + d);
         ws_load<NX>(p.x + sg.off + sg.cstart, sg.len - sg.cstart, slots, lane);
         ws_set(p, ws, sg, lane);
         ws_segment_df<NX>(p, base, lane);
@@ -501,7 +740,7 @@ __global__ void __launch_bounds__(kWsThreads, ws_ctas_per_sm<N>())
     // ---- the others ----
     if (d < total) {
         {
-            const SegGeom sg = seg_geom<WC::kGroup>(p, d);
+            const SegGeom sg = seg_geom<WC::kGroup>(p, skip + d);
             // the first group is on its way while the next segment is looked up
             if (sg.K > 0) ws_load<N>(p.x + sg.off + sg.cstart, sg.len - sg.cstart, slots, lane);
             if (lane == 0) ws.cur = 0;
@@ -515,7 +754,7 @@ __global__ void __launch_bounds__(kWsThreads, ws_ctas_per_sm<N>())
                 const int64_t dn = next();
                 SegGeom nx;
                 nx.K = 0;
-                if (dn < ws.total) nx = seg_geom<WC::kGroup>(p, dn);
+                if (dn < ws.total) nx = seg_geom<WC::kGroup>(p, skip + dn);
                 if (lane == 0) {
                     ws.next = dn;
                     ws.nbase = nx.K > 0 ? nx.off + nx.cstart : -1;
@@ -526,7 +765,7 @@ __global__ void __launch_bounds__(kWsThreads, ws_ctas_per_sm<N>())
             ws_run_segment<N, CRK>(p, base, lane);
             const int64_t dn = ws.next;
             if (dn >= ws.total) break;
-            const SegGeom sg = seg_geom<WC::kGroup>(p, dn);
+            const SegGeom sg = seg_geom<WC::kGroup>(p, skip + dn);
             __syncwarp();
             ws_set(p, ws, sg, lane);
         }
