@@ -35,6 +35,22 @@ def _check_device(t: torch.Tensor, name: str):
         raise ValueError(f"{name} must be a CUDA tensor (this library has no CPU path)")
 
 
+def _stream(device: torch.device) -> int:
+    """The current stream of a CUDA device as an integer handle."""
+    index = device.index
+    return torch._C._cuda_getCurrentRawStream(
+        torch.cuda.current_device() if index is None else index)
+
+
+def _lengths(lengths) -> tuple:
+    if type(lengths) in (list, tuple):
+        try:
+            return tuple(map(int, lengths))
+        except (TypeError, ValueError):
+            pass  # nested, or tensors of several values
+    return tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
+
+
 class SosFilter:
     """A reusable plan: channel lengths, section count and tuning fixed;
     signals, coefficients and states passed per call."""
@@ -58,6 +74,9 @@ class SosFilter:
         self.kmax = int(kmax)
         self.total = int(lh.sum())
         self.tuning = tuple(tuning) if tuning is not None else (0, 0, 0, 0)
+        # every channel with all kmax sections, for calls that give no K (copied
+        # from the host: complete before any stream can use it)
+        self._all = torch.full((self.n_channels,), self.kmax, dtype=torch.int32).to(self.device)
         nbytes = _abi.sos_workspace_size(self.n_channels, self.kmax, lh.data_ptr(), self.tuning)
         if nbytes == 0:
             raise ValueError("unsupported sizes or tuning %r" % (self.tuning,))
@@ -75,22 +94,24 @@ class SosFilter:
         _check_device(x, "x")
         if x.dtype != torch.float32 or not x.is_contiguous() or x.numel() != self.total:
             raise ValueError("x must be contiguous float32 with sum(lengths) elements")
-        sos = sos.reshape(C, kmax, 6)
+        if sos.shape != (C, kmax, 6):
+            sos = sos.reshape(C, kmax, 6)
         if sos.dtype != torch.float64 or not sos.is_contiguous() or sos.device != x.device:
             raise ValueError("sos must be contiguous float64 [C, kmax, 6] on x's device")
         if K is None:
-            K = torch.full((C,), kmax, dtype=torch.int32, device=x.device)
+            K = self._k_all(x.device)
         if K.dtype != torch.int32 or not K.is_contiguous() or K.numel() != C:
             raise ValueError("K must be contiguous int32 [C]")
         if zi is not None:
-            zi = zi.reshape(C, kmax, 2)
+            if zi.shape != (C, kmax, 2):
+                zi = zi.reshape(C, kmax, 2)
             if zi.dtype != torch.float32 or not zi.is_contiguous():
                 raise ValueError("zi must be contiguous float32 [C, kmax, 2]")
         if y is None:
             y = torch.empty_like(x)
         if zf is None and want_zf:
             zf = torch.empty((C, kmax, 2), dtype=torch.float32, device=x.device)
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_filter(x.data_ptr(), sos.data_ptr(), K.data_ptr(), C, kmax,
                              self.lengths.data_ptr(), self.lengths_host.data_ptr(),
                              zi.data_ptr() if zi is not None else 0, y.data_ptr(),
@@ -99,6 +120,9 @@ class SosFilter:
         if st != 0:
             raise SosError(st, "sos_filter")
         return y, zf
+
+    def _k_all(self, device: torch.device) -> torch.Tensor:
+        return self._all if device == self._all.device else self._all.to(device)
 
     def prepare(self, sos: torch.Tensor, K: Optional[torch.Tensor] = None):
         """Enqueue only the plan kernel (coefficient tables) for these sos/K."""
@@ -118,7 +142,7 @@ class SosFilter:
               zf: Optional[torch.Tensor] = None):
         """Enqueue only the filtering kernel, using the tables of the last
         prepare() on this plan."""
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_apply(x.data_ptr(), self.n_channels, self.kmax, self.lengths_host.data_ptr(),
                             zi.data_ptr() if zi is not None else 0, y.data_ptr(),
                             zf.data_ptr() if zf is not None else 0, self.workspace.data_ptr(),
@@ -135,7 +159,7 @@ class SosFilter:
         C, kmax = self.n_channels, self.kmax
         sos = sos.reshape(C, kmax, 6).contiguous()
         if K is None:
-            K = torch.full((C,), kmax, dtype=torch.int32, device=x.device)
+            K = self._k_all(x.device)
         if not hasattr(self, "_bws"):
             nb = _abi.sos_backward_workspace_size(C, kmax, self.lengths_host.data_ptr(),
                                                   self.tuning)
@@ -150,7 +174,7 @@ class SosFilter:
         gsos = torch.empty((C, kmax, 6), dtype=torch.float64, device=x.device)
         gzi = torch.empty((C, kmax, 2), dtype=torch.float32, device=x.device) if want_zi else None
         gzf = grad_zf.reshape(C, kmax, 2).contiguous() if grad_zf is not None else None
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_filter_backward(x.data_ptr(), sos.data_ptr(), K.data_ptr(), C, kmax,
                                       self.lengths.data_ptr(), self.lengths_host.data_ptr(),
                                       zi.data_ptr() if zi is not None else 0, grad_y.data_ptr(),
@@ -200,10 +224,10 @@ class SosFilter:
             raise ValueError("x must be contiguous float32 with sum(lengths) elements")
         sos = sos.reshape(C, kmax, 6).contiguous()
         if K is None:
-            K = torch.full((C,), kmax, dtype=torch.int32, device=x.device)
+            K = self._k_all(x.device)
         y = torch.empty_like(x) if y is None else y
         tmp = torch.empty_like(x) if tmp is None else tmp
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_filtfilt(x.data_ptr(), sos.data_ptr(), K.data_ptr(), C, kmax,
                                self.lengths.data_ptr(), self.lengths_host.data_ptr(), y.data_ptr(),
                                tmp.data_ptr(), self.workspace.data_ptr(), self.ws_bytes, self.tuning,
@@ -217,7 +241,7 @@ class SosFilter:
         """The comparison algorithms on this plan's tables: "scalar" or
         "block" filtering (sos_apply_baseline), segments of seg_len."""
         algo = {"scalar": 0, "block": 1}[algorithm]
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_apply_baseline(algo, x.data_ptr(), self.n_channels, self.kmax,
                                      self.lengths_host.data_ptr(),
                                      zi.data_ptr() if zi is not None else 0, y.data_ptr(),
@@ -240,7 +264,7 @@ class SosFilter:
     def apply_part(self, part: str, x: torch.Tensor, y: torch.Tensor,
                    zi: Optional[torch.Tensor] = None, zf: Optional[torch.Tensor] = None):
         """One of the two launches of apply(): "pipeline" or "carried"."""
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         st = _abi.sos_apply_part(part, x.data_ptr(), self.n_channels, self.kmax,
                                  self.lengths_host.data_ptr(),
                                  zi.data_ptr() if zi is not None else 0, y.data_ptr(),
@@ -308,7 +332,7 @@ class SosStream:
             raise ValueError("x must be contiguous float32 [C, chunk]")
         if y is None:
             y = torch.empty_like(x)
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x.device)
         zi, zf = self._bufs[self._cur], self._bufs[1 - self._cur]
         flags = _abi.SOS_STREAM_FOREIGN_STATE if self._foreign else 0
         st = _abi.sos_stream(x.data_ptr(), y.data_ptr(), zi.data_ptr(), zf.data_ptr(),
@@ -350,7 +374,7 @@ def sosfilt(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] = None
             raise ValueError("tuning must be a 4-tuple, None or 'auto'")
         from .autotune import autotune
         tuning = autotune(x, sos, K, lengths, zi)
-    lh = tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
+    lh = _lengths(lengths)
     key = (x.device, lh, kmax, tuple(tuning) if tuning is not None else None)
     plan = _plans.get(key)
     if plan is None:
@@ -457,7 +481,7 @@ def sosfilt_host(x_host: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tens
         if C != 1:
             raise ValueError("lengths are required for more than one channel")
         lengths = [x_host.numel()]
-    lh = tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
+    lh = _lengths(lengths)
     key = (sos.device, lh, kmax, tuple(tuning) if tuning is not None else None, int(block))
     plan = _host_plans.get(key)
     if plan is None:
@@ -508,7 +532,7 @@ def sosfiltfilt(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] = 
         if C != 1:
             raise ValueError("lengths are required for more than one channel")
         lengths = [x.numel()]
-    lh = tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
+    lh = _lengths(lengths)
     key = (x.device, lh, kmax, tuple(tuning) if tuning is not None else None)
     plan = _plans.get(key)
     if plan is None:
@@ -529,7 +553,7 @@ def sosfilt_diff(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] =
         if C != 1:
             raise ValueError("lengths are required for more than one channel")
         lengths = [x.numel()]
-    lh = tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
+    lh = _lengths(lengths)
     key = (x.device, lh, kmax, tuple(tuning) if tuning is not None else None)
     plan = _plans.get(key)
     if plan is None:
@@ -538,7 +562,7 @@ def sosfilt_diff(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] =
             _plans.clear()
         _plans[key] = plan
     if K is None:
-        K = torch.full((C,), kmax, dtype=torch.int32, device=x.device)
+        K = plan._k_all(x.device)
     if zi is not None:
         zi = zi.reshape(C, kmax, 2)
     return SosFilterFunction.apply(x, sos3, zi, plan, K)

@@ -8,6 +8,7 @@ fallback implementation.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 import threading
 
@@ -55,6 +56,8 @@ def load(build_if_missing: bool = False):
     """The loaded library.  Raises if it has not been built (call
     ``paper_2607_14054_gb300.build.build()`` / ``__graft_entry__.build()``)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -119,13 +122,19 @@ def load(build_if_missing: bool = False):
         return lib
 
 
+@functools.lru_cache(maxsize=256)
+def _tuning_ref(n: int, w: int, a: int, f: int):
+    # the library only reads the structure: one per set of values serves every call
+    return ctypes.byref(sos_tuning(n, w, a, f))
+
+
 def _tuning(t):
     if t is None:
         return None
     if isinstance(t, sos_tuning):
         return ctypes.byref(t)
-    n, w, a, f = (list(t) + [0, 0, 0, 0])[:4]
-    return ctypes.byref(sos_tuning(int(n), int(w), int(a), int(f)))
+    n, w, a, f = t if len(t) == 4 else (list(t) + [0, 0, 0, 0])[:4]
+    return _tuning_ref(int(n), int(w), int(a), int(f))
 
 
 def sos_workspace_size(n_channels: int, kmax: int, lengths_host_ptr: int, tuning=None) -> int:
@@ -140,10 +149,9 @@ def sos_workspace_init(ws_ptr: int, ws_bytes: int, stream: int) -> int:
 def sos_filter(x, sos, K, n_channels, kmax, lengths, lengths_host, zi, y, zf, ws, ws_bytes,
                tuning, stream) -> int:
     """All pointer arguments are integers (0 for NULL)."""
-    V = ctypes.c_void_p
-    return int(load().sos_filter(V(x), V(sos), V(K), n_channels, kmax, V(lengths), V(lengths_host),
-                                 V(zi or None), V(y), V(zf or None), V(ws), ws_bytes,
-                                 _tuning(tuning), V(stream)))
+    return int(load().sos_filter(x, sos, K, n_channels, kmax, lengths, lengths_host,
+                                 zi or None, y, zf or None, ws, ws_bytes,
+                                 _tuning(tuning), stream))
 
 
 def sos_filter_host_sizes(n_channels, kmax, lengths_host, block, tuning):
@@ -160,24 +168,21 @@ def sos_filter_host_sizes(n_channels, kmax, lengths_host, block, tuning):
 def sos_filter_host(x_host, sos, K, n_channels, kmax, lengths, lengths_host, zi, y_host, zf, ws,
                     ws_bytes, staging, staging_bytes, block, tuning, stream) -> int:
     """All pointer arguments are integers (0 for NULL); x_host, y_host host."""
-    V = ctypes.c_void_p
-    return int(load().sos_filter_host(V(x_host), V(sos), V(K), n_channels, kmax, V(lengths),
-                                      V(lengths_host), V(zi or None), V(y_host), V(zf or None),
-                                      V(ws), ws_bytes, V(staging), staging_bytes, int(block),
-                                      _tuning(tuning), V(stream)))
+    return int(load().sos_filter_host(x_host, sos, K, n_channels, kmax, lengths,
+                                      lengths_host, zi or None, y_host, zf or None,
+                                      ws, ws_bytes, staging, staging_bytes, int(block),
+                                      _tuning(tuning), stream))
 
 
 def sos_prepare(sos, K, n_channels, kmax, lengths, lengths_host, ws, ws_bytes, tuning,
                 stream) -> int:
-    V = ctypes.c_void_p
-    return int(load().sos_prepare(V(sos), V(K), n_channels, kmax, V(lengths), V(lengths_host),
-                                  V(ws), ws_bytes, _tuning(tuning), V(stream)))
+    return int(load().sos_prepare(sos, K, n_channels, kmax, lengths, lengths_host,
+                                  ws, ws_bytes, _tuning(tuning), stream))
 
 
 def sos_apply(x, n_channels, kmax, lengths_host, zi, y, zf, ws, ws_bytes, tuning, stream) -> int:
-    V = ctypes.c_void_p
-    return int(load().sos_apply(V(x), n_channels, kmax, V(lengths_host), V(zi or None), V(y),
-                                V(zf or None), V(ws), ws_bytes, _tuning(tuning), V(stream)))
+    return int(load().sos_apply(x, n_channels, kmax, lengths_host, zi or None, y,
+                                zf or None, ws, ws_bytes, _tuning(tuning), stream))
 
 
 def sos_apply_part(part: str, x, n_channels, kmax, lengths_host, zi, y, zf, ws, ws_bytes,
@@ -213,10 +218,9 @@ def sos_apply_baseline(algorithm, x, n_channels, kmax, lengths_host, zi, y, zf, 
 def sos_filtfilt(x, sos, K, n_channels, kmax, lengths, lengths_host, y, tmp, ws, ws_bytes, tuning,
                  stream) -> int:
     """All pointer arguments are integers."""
-    V = ctypes.c_void_p
-    return int(load().sos_filtfilt(V(x), V(sos), V(K), n_channels, kmax, V(lengths),
-                                   V(lengths_host), V(y), V(tmp), V(ws), ws_bytes, _tuning(tuning),
-                                   V(stream)))
+    return int(load().sos_filtfilt(x, sos, K, n_channels, kmax, lengths,
+                                   lengths_host, y, tmp, ws, ws_bytes, _tuning(tuning),
+                                   stream))
 
 
 SOS_STREAM_FOREIGN_STATE = 1
@@ -225,10 +229,9 @@ SOS_STREAM_FOREIGN_STATE = 1
 def sos_stream(x, y, zi, zf, n_channels, kmax, chunk, flags, ws, ws_bytes, tuning,
                stream) -> int:
     """All pointer arguments are integers (0 for NULL)."""
-    V = ctypes.c_void_p
-    return int(load().sos_stream(V(x), V(y), V(zi or None), V(zf or None), n_channels, kmax,
-                                 int(chunk), int(flags), V(ws), ws_bytes, _tuning(tuning),
-                                 V(stream)))
+    return int(load().sos_stream(x, y, zi or None, zf or None, n_channels, kmax,
+                                 int(chunk), int(flags), ws, ws_bytes, _tuning(tuning),
+                                 stream))
 
 
 def sos_device_status(ws_ptr: int, stream: int) -> int:
@@ -245,12 +248,11 @@ def sos_backward_workspace_size(n_channels: int, kmax: int, lengths_host_ptr: in
 def sos_filter_backward(x, sos, K, n_channels, kmax, lengths, lengths_host, zi, grad_y, grad_zf,
                         grad_x, grad_sos, grad_zi, ws, ws_bytes, tuning, stream) -> int:
     """All pointer arguments are integers (0 for NULL)."""
-    V = ctypes.c_void_p
-    return int(load().sos_filter_backward(V(x), V(sos), V(K), n_channels, kmax, V(lengths),
-                                          V(lengths_host), V(zi or None), V(grad_y),
-                                          V(grad_zf or None), V(grad_x), V(grad_sos),
-                                          V(grad_zi or None), V(ws), ws_bytes, _tuning(tuning),
-                                          V(stream)))
+    return int(load().sos_filter_backward(x, sos, K, n_channels, kmax, lengths,
+                                          lengths_host, zi or None, grad_y,
+                                          grad_zf or None, grad_x, grad_sos,
+                                          grad_zi or None, ws, ws_bytes, _tuning(tuning),
+                                          stream))
 
 
 def sos_plan_query(ws_ptr: int, first: int, count: int, horizon_ptr: int, tiles_ptr: int,

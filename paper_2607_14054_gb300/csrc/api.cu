@@ -241,15 +241,8 @@ namespace {
 // which of the two filtering launches a call enqueues
 enum ApplyParts { kPartPipe = 1, kPartCarry = 2 };
 
-sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
-                       const int64_t* lengths_host, const float* zi, float* y, float* zf,
-                       void* workspace, size_t ws_bytes, const sos_tuning* tuning, void* stream,
-                       int parts, bool reversed = false) {
-    Params p{};
-    int64_t tiles = 0, total = 0;
-    const sos_status s = setup(n_channels, kmax, lengths_host, workspace, ws_bytes, tuning, &p,
-                               &tiles, &total);
-    if (s != SOS_OK) return s;
+// x and y given and apart
+sos_status check_signals(const float* x, const float* y, int64_t total) {
     if (total > 0 && (!x || !y)) return SOS_ERR_ARG;
     if (x && y && total > 0) {
         const char* xb = reinterpret_cast<const char*>(x);
@@ -257,6 +250,13 @@ sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
         const size_t bytes = sizeof(float) * (size_t)total;
         if (xb < yb + bytes && yb < xb + bytes) return SOS_ERR_ARG;  // no overlap
     }
+    return SOS_OK;
+}
+
+// the launches of one pass over a call that setup() has filled p for
+sos_status enqueue_apply(Params p, int64_t tiles, const float* x, const float* zi, float* y,
+                         float* zf, void* stream, int parts, bool reversed) {
+    const int64_t total = p.total;
     p.x = x;
     p.y = y;
     p.zi = zi;
@@ -287,6 +287,19 @@ sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
         if (launch_forward(p, launch_tiles, st, early) != cudaSuccess) return SOS_ERR_CUDA;
     }
     return SOS_OK;
+}
+
+sos_status apply_parts(const float* x, int32_t n_channels, int32_t kmax,
+                       const int64_t* lengths_host, const float* zi, float* y, float* zf,
+                       void* workspace, size_t ws_bytes, const sos_tuning* tuning, void* stream,
+                       int parts) {
+    Params p{};
+    int64_t tiles = 0, total = 0;
+    sos_status s = setup(n_channels, kmax, lengths_host, workspace, ws_bytes, tuning, &p, &tiles,
+                         &total);
+    if (s == SOS_OK) s = check_signals(x, y, total);
+    if (s != SOS_OK) return s;
+    return enqueue_apply(p, tiles, x, zi, y, zf, stream, parts, false);
 }
 
 }  // namespace
@@ -320,25 +333,20 @@ sos_status sos_filter(const float* x, const double* sos, const int32_t* K, int32
                       int32_t kmax, const int64_t* lengths, const int64_t* lengths_host,
                       const float* zi, float* y, float* zf, void* workspace, size_t ws_bytes,
                       const sos_tuning* tuning, void* stream) {
-    // check everything the second half checks before enqueuing the first
+    // everything is checked before the first launch
     Params p{};
     int64_t tiles = 0, total = 0;
     sos_status s = setup(n_channels, kmax, lengths_host, workspace, ws_bytes, tuning, &p, &tiles,
                          &total);
     if (s != SOS_OK) return s;
     if (!sos || !K || !lengths) return SOS_ERR_ARG;
-    if (total > 0 && (!x || !y)) return SOS_ERR_ARG;
-    if (x && y && total > 0) {
-        const char* xb = reinterpret_cast<const char*>(x);
-        const char* yb = reinterpret_cast<const char*>(y);
-        const size_t bytes = sizeof(float) * (size_t)total;
-        if (xb < yb + bytes && yb < xb + bytes) return SOS_ERR_ARG;
-    }
-    s = sos_prepare(sos, K, n_channels, kmax, lengths, lengths_host, workspace, ws_bytes, tuning,
-                    stream);
+    s = check_signals(x, y, total);
     if (s != SOS_OK) return s;
-    return sos_apply(x, n_channels, kmax, lengths_host, zi, y, zf, workspace, ws_bytes, tuning,
-                     stream);
+    p.sos = sos;
+    p.K = K;
+    p.lengths = lengths;
+    if (launch_plan(p, static_cast<cudaStream_t>(stream)) != cudaSuccess) return SOS_ERR_CUDA;
+    return enqueue_apply(p, tiles, x, zi, y, zf, stream, kPartPipe | kPartCarry, false);
 }
 
 sos_status sos_stream(const float* x, float* y, const float* zi, float* zf, int32_t n_channels,
@@ -447,14 +455,13 @@ sos_status sos_filtfilt(const float* x, const double* sos, const int32_t* K, int
     }
     // two forward passes from zero state, each writing its output
     // time-reversed: y = R H R H x
-    s = sos_prepare(sos, K, n_channels, kmax, lengths, lengths_host, workspace, ws_bytes, tuning,
-                    stream);
+    p.sos = sos;
+    p.K = K;
+    p.lengths = lengths;
+    if (launch_plan(p, static_cast<cudaStream_t>(stream)) != cudaSuccess) return SOS_ERR_CUDA;
+    s = enqueue_apply(p, tiles, x, nullptr, tmp, nullptr, stream, kPartPipe | kPartCarry, true);
     if (s != SOS_OK) return s;
-    s = apply_parts(x, n_channels, kmax, lengths_host, nullptr, tmp, nullptr, workspace, ws_bytes,
-                    tuning, stream, kPartPipe | kPartCarry, true);
-    if (s != SOS_OK) return s;
-    return apply_parts(tmp, n_channels, kmax, lengths_host, nullptr, y, nullptr, workspace,
-                       ws_bytes, tuning, stream, kPartPipe | kPartCarry, true);
+    return enqueue_apply(p, tiles, tmp, nullptr, y, nullptr, stream, kPartPipe | kPartCarry, true);
 }
 
 sos_status sos_device_status(void* workspace, void* stream) {
