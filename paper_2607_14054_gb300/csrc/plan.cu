@@ -517,8 +517,8 @@ __device__ float handoff_error(const double (*rows)[5], const float (*rowsf)[5],
 // horizon, but it holds for repeated poles.  tz: the same for the response
 // of a unit initial state (it enters a section's recursion like an impulse
 // of at most unit size, so B_k is taken as at least 1).  -1 where r >= 1 or
-// no such P below 2^30.  One thread.
-__device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int& tz) {
+// no such P below 2^30.  One warp, the same result in every lane.
+__device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int lane, int& tz) {
     tz = -1;
     if (K < 1 || !(h2 > 0.f)) return -1;
     double r = 0.0, logA = 0.0, logAs = 0.0;
@@ -543,23 +543,36 @@ __device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int& t
         tz = ((2 * K + 1) + 15) / 16 * 16;
         return tz;
     }
-    const double m = 2.0 * K, lr = log(r);
+    const double m = 2.0 * K, lr = log(r), lgm = lgamma(m);
     const double target = log((double)kHorizonEps * (double)h2);
     // the first n past the peak (ratio < 1) where the log tail bound with
     // prefactor log a is below the target, in multiples of 16; -1 if none
     auto first = [&](double loga) -> int {
+        // (n + m - 1)! / n! = (n + 1) .. (n + m - 1): at most 15 factors below 2^31
         auto tail = [&](double n) {
             const double ratio = r * (n + m) / (n + 1.0);
-            return loga + lgamma(n + m) - lgamma(m) - lgamma(n + 1.0) + n * lr - log1p(-ratio);
+            double pr = 1.0;
+            for (int i = 1; i < 2 * K; ++i) pr *= n + i;
+            return loga + log(pr) - lgm + n * lr - log1p(-ratio);
         };
         double lo = fmax(ceil((m * r - 1.0) / (1.0 - r)) + 1.0, m);
         double hi = 1073741824.0;
+        // (the same in every lane) hi satisfies the bound, lo does not; the
+        // lanes try 32 points between them at a time, where one thread's
+        // bisection took 30 steps of FP64 log-gammas (plan of 4096 channels,
+        // the resonant ones of which come here: 620 -> 406 us)
         if (!(tail(hi) <= target)) return -1;
         if (tail(lo) <= target) hi = lo;
-        for (int it = 0; it < 40 && hi - lo > 1.0; ++it) {
-            const double mid = floor(0.5 * (lo + hi));
-            if (tail(mid) <= target) hi = mid;
-            else lo = mid;
+        while (hi - lo > 1.0) {
+            const double w = hi - lo;
+            const double t = floor(lo + w * ((lane + 1) / 33.0));
+            const bool ok = t > lo && t < hi && tail(t) <= target;
+            const unsigned yes = __ballot_sync(0xffffffffu, ok);
+            const unsigned no = __ballot_sync(0xffffffffu, t > lo && t < hi && !ok);
+            if (yes) hi = __shfl_sync(0xffffffffu, t, __ffs(yes) - 1);
+            const unsigned below = yes ? no & ((1u << (__ffs(yes) - 1)) - 1u) : no;
+            if (below) lo = __shfl_sync(0xffffffffu, t, 31 - __clz(below));
+            if (!(hi - lo < w)) break;
         }
         const int64_t n = ((int64_t)hi + 15) / 16 * 16;
         return n < (int64_t)1 << 30 ? (int)n : -1;
@@ -907,9 +920,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         // for at least eight segments (the look-back is faster below that)
         if (P < 0 && !carry_only && Kc > 0) {
             int Pf = -1, tzf = -1;
-            if (lane == 0) Pf = horizon_fallback(s_row, Kc, s_h2, tzf);
-            Pf = __shfl_sync(0xffffffffu, Pf, 0);
-            tzf = __shfl_sync(0xffffffffu, tzf, 0);
+            Pf = horizon_fallback(s_row, Kc, s_h2, lane, tzf);
             const int64_t want = Pf >= 0 ? (2LL * Pf > tzf ? 2LL * Pf : (int64_t)tzf) : 0;
             const int64_t lenc = p.lengths[c];
             if (Pf >= 0 && ((p.flags_opt & kFlagBackwardPlan) || lenc >= 8 * want)) {
