@@ -574,7 +574,7 @@ sos_status sos_plan_recomputed(void* workspace, int32_t* channels, void* stream)
 
 namespace sosf {
 cudaError_t launch_adjoint(const Params& p, int sms, double* grad_sos, cudaStream_t stream);
-int64_t adjoint_warps(int N, int sms);
+int64_t adjoint_segments(int N, int sms);
 int64_t adjoint_ck_slots(int N, int64_t total_len, int32_t C);
 }  // namespace sosf
 
@@ -599,16 +599,16 @@ BwdLayout bwd_layout(size_t base, int32_t C, int32_t kmax, int64_t total_len, in
 }
 
 // Backward segment length, in whole groups (at least 8, at most 64): from
-// the call's samples over the adjoint kernel's resident warps upwards, the
+// the call's samples over the adjoint kernel's resident CTAs upwards, the
 // length whose segments (whole channels cut at it) take the fewest group
-// steps on the warps, rounds x groups per segment, so that a channel's last
-// partial segment does not start a second round on a few warps; a horizon
+// steps on the CTAs, rounds x groups per segment, so that a channel's last
+// partial segment does not start a second round on a few CTAs; a horizon
 // of up to half a segment fits.
 int64_t backward_segment_length(const int64_t* lengths_host, int32_t C, int64_t total_len,
                                 int N) {
     const int64_t group = 32LL * N;
     const int sms = device_sms() > 0 ? device_sms() : 148;
-    int64_t units = adjoint_warps(N, sms);
+    int64_t units = adjoint_segments(N, sms);
     if (units < 1) units = 1;
     int64_t g0 = (total_len + units * group - 1) / (units * group);
     if (g0 < 8) g0 = 8;
