@@ -352,9 +352,10 @@ def end_to_end(P, x, sos, stream, samples, world, args, tuning):
 # the kernel for channels within their memory horizon: its committed ncu
 # summary and the sources it is built from
 _COMMON_SOURCES = ["pipe_section.cuh", "sos_pipe.cuh", "sos_async.cuh", "sos_kernels.cuh",
-                   "sos_common.cuh"]
+                   "sos_common.cuh", "sos_f2.cuh"]
 KERNEL_PROFILES = {
-    "sos_warpseg_kernel": ("sos_warpseg_kernel_bp16_2e24.json", ["warpseg.cu"] + _COMMON_SOURCES),
+    "sos_warpseg_kernel": ("sos_warpseg_kernel_bp16_2e24.json", ["warpseg.cu", "warpseg.cuh", "warpseg_n16.cu", "warpseg_n32.cu",
+                            "warpseg_n64.cu", "long_section.cuh"] + _COMMON_SOURCES),
     "sos_pipe_kernel": ("sos_pipe_kernel_bp16_2e24.json", ["pipe.cu"] + _COMMON_SOURCES),
 }
 

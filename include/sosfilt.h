@@ -66,9 +66,10 @@ typedef enum sos_status {
 
 /* Tuning knobs.  Pass NULL for the library defaults.
  *   n_blocks: N, samples per lane per group (the paper's number of blocks):
- *             16, 32 or 64 (0 = default 32).
+ *             16, 32 or 64 (0 = default: 64 for the filter, 32 for the
+ *             backward, the stream's own choice by block size).
  *   warps:    W, warps per tile (one tile = W*32*N samples): 4, 8 or 16
- *             (0 = default 8).
+ *             (0 = default: 4 with the default N, else 8; the backward 8).
  *   algo:     recursive-stage solver: 0 = default (PH), 1 = PH (Sec. VI-B),
  *             2 = cyclic reduction (Sec. VI-C) for every section whose
  *             reduction is well conditioned (max |f_i / e_i| <= 100 over the
@@ -99,7 +100,7 @@ typedef enum sos_status {
  *             sos_prepare; same results, for timing the full plan).
  *             bit 4 (SOS_FLAG_DOUBLE_FLOAT): run every channel within its
  *             memory horizon with double-float samples (precision class 3
- *             of sos_plan_extended), whatever the plan's estimate; about ten
+ *             of sos_plan_extended), whatever the plan's estimate; about five
  *             times the arithmetic, for results within about 2^-40 of the
  *             exact ones where FP32 would lose digits.
  *             bits 8..11 (SOS_FLAG_WS_CTAS(n)): CTAs per SM of the
@@ -111,10 +112,13 @@ typedef enum sos_status {
  * Cross-tile state.  The plan bounds each channel's impulse-response tail by
  * partial fractions over its poles and finds its memory horizon P: the warm-up
  * after which the state a tile would drop changes the output by less than
- * 2^-30 relative.  The channel is then cut into segments of S samples (the
- * call's segment length, a multiple of 32 N chosen from its total length, or
- * 2 P rounded up to whole groups when that is longer) that each start P
- * samples early from zero state (no cross-segment dependency).  Coincident
+ * 2^-30 relative.  The channel is then cut into segments (by default of the
+ * length whose computed samples, warm-up included, keep the launch's warps
+ * busy for the shortest time, set per channel from the horizons of all; the
+ * tile counts sos_plan_query reports stay those of segments of at least 2 P)
+ * that each start P samples early from zero state (no cross-segment
+ * dependency).  Channels with P > 8192 keep segments of 2 P and have each run
+ * by a team of up to four warps, one per share of the sections.  Coincident
  * poles, where partial fractions fail, get a cruder bound over the largest
  * pole radius r (a tail of the form C(n + 2K - 1, 2K - 1) r^n) when the
  * channel is at least eight of the segments it asks for.  Where no horizon is
@@ -423,9 +427,12 @@ sos_status sos_plan_query(void *workspace, int32_t first, int32_t count, int32_t
  *   1  some section's in-lane recursions add the low parts of a1, a2 (FP32
  *      rounding of a1, a2 displaces its poles by more than 2^-18 of their
  *      distance to the unit circle);
- *   2  some section also runs its lane scan and fold (S4) in double-float
- *      (the largest entry of its transition powers A^(N 2^j), A^(N l) exceeds
- *      8, or the displacement exceeds 1e-4);
+ *   2  some section has poles close to z = +-1 (the largest entry of its
+ *      transition powers A^(N 2^j), A^(N l) exceeds 8, taken at N = 32 for
+ *      N = 64) or a displacement beyond 1e-4: its scan state is kept in a
+ *      basis in which those powers are small (s1 = z1, s2 = (z2 - a1 z1 / 2) /
+ *      w), and channels with P > 8192 run the scan and fold (S4) in
+ *      double-float;
  *   3  sections run with double-float samples (about 44 bits): the plan's
  *      estimate of the error that FP32 rounding of the signal handed from
  *      section k to k + 1 would cause at the output (white input, from the

@@ -204,9 +204,8 @@ class SosFilter:
         return h, t
 
     def plan_extended(self):
-        """Per channel, 1 where some section is ill-conditioned for FP32 and
-        the default kernel runs its lane scan in extended precision (int32
-        host tensor, from the latest prepare)."""
+        """Per channel its precision class 0..3 (sos_plan_extended; int32 host
+        tensor, from the latest prepare)."""
         e = torch.empty(self.n_channels, dtype=torch.int32)
         stream = torch.cuda.current_stream(self.device).cuda_stream
         st = _abi.sos_plan_extended(self.workspace.data_ptr(), 0, self.n_channels, e.data_ptr(),
