@@ -1148,14 +1148,16 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
                 far->phi_lo[lane] = to_f4_lo(pow2(lane));
             }
         }
-        if (ext_n(N) != N &&
-            !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE))) {
+        if (ext_n(N) != N && !(p.flags_opt & kFlagBackwardPlan)) {
             // a channel of precision class 3 runs with ext_n(N) = N/2 samples
-            // per lane: its powers again, one squaring earlier
+            // per lane on the warp-segment and streaming kernels: its powers
+            // again, one squaring earlier, beside phi_c (a stream's plan may
+            // carry the section pipeline's flag, whose kernel takes N)
             asm volatile("bar.sync 4, %0;" ::"r"(32 * Kc) : "memory");
             if (s_ext >= 3 && lane < 7)
-                out32->phi_c[lane] = scan_basis(lane < 5 ? pow2(lane) : s_part[k][lane - 4], a1,
-                                                scan_scale(a1, a2));
+                reinterpret_cast<LongCoef*>(outdf)->phi_x[lane] =
+                    scan_basis(lane < 5 ? pow2(lane) : s_part[k][lane - 4], a1,
+                               scan_scale(a1, a2));
         }
         return true;
     }

@@ -126,7 +126,8 @@ constexpr int32_t kFlagBackwardPlan = 1 << 16;
 
 // Samples per lane of a precision class 3 channel on the warp-segment and
 // streaming kernels: its double-float code needs the registers that a chunk
-// of 64 would take (the plan builds such a channel's powers for this N).
+// of 64 would take (the plan builds such a channel's powers for this N beside
+// the others, LongCoef::phi_x).
 __host__ __device__ constexpr int ext_n(int N) { return N == 64 ? 32 : N; }
 
 // Per (channel, section) FP32 coefficients and transition-matrix powers.
@@ -218,11 +219,15 @@ struct __align__(16) CoefDF {
     float4 theta_hi[18][2];
 };
 
-// In its place for long-memory channels, which are never carried by the
-// look-back: the low parts of phi_pow and lane_pow.
+// In its place for channels within their memory horizon, which are never
+// carried by the look-back.  Long-memory channels: the low parts of phi_pow and
+// lane_pow.  Channels of precision class 3 at N != ext_n(N): phi_c for ext_n(N)
+// samples per lane (phi_c itself is for N in every plan, whichever kernel reads
+// it).
 struct __align__(16) LongCoef {
     float4 phi_lo[5];
     float4 lane_lo[32];
+    float4 phi_x[7];
 };
 static_assert(sizeof(LongCoef) <= sizeof(CoefDF), "LongCoef lies in CoefDF's place");
 

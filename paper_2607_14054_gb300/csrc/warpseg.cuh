@@ -137,11 +137,15 @@ __device__ __forceinline__ SecDF load_secdf(const Coef32* cf) {
                  df{br.z, bl.z}};
 }
 
-// the copies of a channel's K sections, one cp.async group
-__device__ __forceinline__ void ws_stage(const Coef32* cf0, int K, WsCoef* sc, int lane) {
+// the copies of a channel's K sections, one cp.async group; cx: where the
+// channel's powers for other than the plan's N samples per lane are, else null
+__device__ __forceinline__ void ws_stage(const Coef32* cf0, const CoefDF* cx, int K, WsCoef* sc,
+                                         int lane) {
     for (int i = lane; i < 10 * K; i += 32) {
         const int k = i / 10, f = i % 10;
         const float4* src = f == 0 ? &cf0[k].ab : f == 1 ? &cf0[k].misc : &cf0[k].phi_c[0] + f - 2;
+        if (cx && f >= 2 && f < 9)
+            src = &reinterpret_cast<const LongCoef*>(cx + k)->phi_x[0] + f - 2;
         cp_async16(reinterpret_cast<float4*>(sc) + i, src);
     }
     cp_async_commit();
@@ -375,7 +379,11 @@ __device__ __forceinline__ void ws_segment(const Params& p, volatile WsSeg& sg, 
     // (scaled by 1/G_k when b0 is factored) on the channel's first segment,
     // zero state after a warm-up
     __syncwarp();
-    if (!CR) ws_stage(p.c32 + (int64_t)sg.c * p.kmax, sg.K, s_ws.cf[ws_warp()], lane);
+    if (!CR) {
+        const int64_t at = (int64_t)sg.c * p.kmax;
+        ws_stage(p.c32 + at, PREC == kPrecDF && p.N != N ? p.cdf + at : nullptr, sg.K,
+                 s_ws.cf[ws_warp()], lane);
+    }
     if (lane < sg.K) {
         const int c = sg.c;
         float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
