@@ -588,9 +588,11 @@ size_t adj_smem(int N) {
 
 // segments (CTAs) of the adjoint kernel resident on the device (0 on error)
 int64_t adjoint_segments(int N, int sms) {
-    static int s_occ[3] = {0, 0, 0};
+    static int s_occ[kDeviceSlots][3] = {};
+    const int dev = device_slot();
+    if (dev < 0) return 0;
     const int idx = N == 16 ? 0 : N == 32 ? 1 : 2;
-    if (s_occ[idx] == 0) {
+    if (s_occ[dev][idx] == 0) {
         if (cudaFuncSetAttribute(adj_fn(N), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)adj_smem(N)) != cudaSuccess)
             return 0;
@@ -598,9 +600,9 @@ int64_t adjoint_segments(int N, int sms) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, adj_fn(N), kBwThreads,
                                                           adj_smem(N)) != cudaSuccess)
             return 0;
-        s_occ[idx] = occ;
+        s_occ[dev][idx] = occ;
     }
-    return (int64_t)sms * s_occ[idx];
+    return (int64_t)sms * s_occ[dev][idx];
 }
 
 // checkpoint slots the adjoint kernel may use (see ck_slot)

@@ -250,12 +250,14 @@ cudaError_t launch_compare(const Params& p, int algo, int64_t seg_len, int64_t m
         sos_scalar_kernel<<<dim3(gx, (unsigned)p.C), threads, 0, stream>>>(p, seg_len);
     } else {
         const size_t smem = sizeof(float) * kBlkWarps * kMaxSections * 64;
-        static bool attr = false;
-        if (!attr) {
+        static bool attr[kDeviceSlots] = {};
+        const int dev = device_slot();
+        if (dev < 0) return cudaErrorInvalidDevice;
+        if (!attr[dev]) {
             const cudaError_t e = cudaFuncSetAttribute(
                 sos_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
-            attr = true;
+            attr[dev] = true;
         }
         const unsigned gx = (unsigned)((max_segs + kBlkWarps - 1) / kBlkWarps);
         sos_block_kernel<<<dim3(gx, (unsigned)p.C), kBlkWarps * 32, smem, stream>>>(p, seg_len);

@@ -264,13 +264,15 @@ cudaError_t launch_pipe(const Params& p, int64_t grid, cudaStream_t stream, bool
                        : (p.N == 16 ? SOSF_PIPE(16, false) : p.N == 32 ? SOSF_PIPE(32, false)
                                                                 : SOSF_PIPE(64, false));
     const size_t smem = 2 * sizeof(float) * 32 * (size_t)(p.N + 4) * kPipeRing;
-    static bool attr[2][3] = {{false, false, false}, {false, false, false}};
+    static bool attr[kDeviceSlots][2][3] = {};
+    const int dev = device_slot();
+    if (dev < 0) return cudaErrorInvalidDevice;
     const int idx = p.N == 16 ? 0 : p.N == 32 ? 1 : 2;
-    if (!attr[z][idx]) {
+    if (!attr[dev][z][idx]) {
         const cudaError_t e =
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        attr[z][idx] = true;
+        attr[dev][z][idx] = true;
     }
     if (grid < 1) return cudaSuccess;
     return launch_params(fn, (grid + 1) / 2, 2 * kPipeThreads, smem, p, stream, early);

@@ -1444,13 +1444,15 @@ cudaError_t launch_plan(const Params& p, cudaStream_t stream) {
     int n = 1;
     while (n < p.C && n < kMaxSortChannels) n <<= 1;
     const size_t smem = p.C <= kMaxSortChannels ? sizeof(unsigned long long) * (size_t)n : 0;
-    static bool attr_set = false;
-    if (!attr_set) {
+    static bool attr_set[kDeviceSlots] = {};
+    const int dev = device_slot();
+    if (dev < 0) return cudaErrorInvalidDevice;
+    if (!attr_set[dev]) {
         const cudaError_t err =
             cudaFuncSetAttribute(plan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(sizeof(unsigned long long) * kMaxSortChannels));
         if (err != cudaSuccess) return err;
-        attr_set = true;
+        attr_set[dev] = true;
     }
     plan_kernel<<<p.C + 1, kPlanThreads, smem, stream>>>(p);
     return cudaGetLastError();

@@ -314,6 +314,15 @@ struct Params {
     int64_t rev;         // 1: each channel's output is written time-reversed (sos_filtfilt)
 };
 
+// Function attributes and occupancy belong to a device: what a launch sets or
+// asks once is kept by device, in arrays of kDeviceSlots.  The current device,
+// -1 where it cannot be told or has no slot.
+constexpr int kDeviceSlots = 64;
+inline int device_slot() {
+    int dev = -1;
+    return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kDeviceSlots ? dev : -1;
+}
+
 // Launch of fn(p); early: programmatic dependent launch, the kernel may be
 // scheduled once the previous kernel in the stream has let it (that kernel
 // executes griddepcontrol.launch_dependents), and waits for that kernel's

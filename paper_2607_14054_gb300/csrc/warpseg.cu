@@ -26,11 +26,13 @@ size_t ws_smem(int N) {
 }  // namespace
 
 // CTAs of the warp-segment kernel (algo 2: the cyclic-reduction one)
-// resident per SM (0 on error)
+// resident per SM of the current device (0 on error)
 int warpseg_ctas_per_sm(int N, int algo) {
-    static int s_occ[2][3] = {{0, 0, 0}, {0, 0, 0}};
+    static int s_occ[kDeviceSlots][2][3] = {};
+    const int dev = device_slot();
+    if (dev < 0) return 0;
     const int idx = N == 16 ? 0 : N == 32 ? 1 : 2, a = algo == 2 ? 1 : 0;
-    if (s_occ[a][idx] == 0) {
+    if (s_occ[dev][a][idx] == 0) {
         const void* fn = ws_fn(N, a == 1);
         // all of the SM's memory as shared memory: with the default split the
         // last of the CTAs that fit may be left for a second wave
@@ -43,9 +45,9 @@ int warpseg_ctas_per_sm(int N, int algo) {
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kWsThreads, ws_smem(N)) !=
             cudaSuccess)
             return 0;
-        s_occ[a][idx] = occ;
+        s_occ[dev][a][idx] = occ;
     }
-    return s_occ[a][idx];
+    return s_occ[dev][a][idx];
 }
 
 int warpseg_warps_per_cta() { return kWsWarps; }
@@ -53,13 +55,15 @@ int warpseg_warps_per_cta() { return kWsWarps; }
 cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32_t maxseg,
                           int32_t foreign, cudaStream_t stream) {
     const void* fn = p.N == 16 ? stream_fn_16() : p.N == 32 ? stream_fn_32() : stream_fn_64();
-    static bool attr[3] = {false, false, false};
+    static bool attr[kDeviceSlots][3] = {};
+    const int dev = device_slot();
+    if (dev < 0) return cudaErrorInvalidDevice;
     const int idx = p.N == 16 ? 0 : p.N == 32 ? 1 : 2;
-    if (!attr[idx]) {
+    if (!attr[dev][idx]) {
         const cudaError_t e =
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws_smem(p.N));
         if (e != cudaSuccess) return e;
-        attr[idx] = true;
+        attr[dev][idx] = true;
     }
     void* args[] = {const_cast<Params*>(&p), &chunk, &seg_len, &maxseg, &foreign};
     const int64_t warps = (int64_t)p.C * maxseg;
