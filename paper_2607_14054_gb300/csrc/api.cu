@@ -30,16 +30,15 @@ struct Tune {
     int N, W, algo, flags;
 };
 
-// The library's defaults: N = 64, W = 4 (tiles of 8,192 samples); N given alone
-// takes W = 8.
+// The library's defaults: N = 64, W = 4 (tiles of 8,192 samples).  N given alone
+// takes W = 8, W given alone N = 32, for which every documented W is compiled.
 bool resolve_tuning(const sos_tuning* t, Tune* out) {
     Tune r{64, 4, 1, 0};
     if (t) {
-        if (t->n_blocks) {
-            r.N = t->n_blocks;
-            r.W = 8;
+        if (t->n_blocks || t->warps) {
+            r.N = t->n_blocks ? t->n_blocks : 32;
+            r.W = t->warps ? t->warps : 8;
         }
-        if (t->warps) r.W = t->warps;
         if (t->algo) r.algo = t->algo;
         r.flags = t->flags;
     }
