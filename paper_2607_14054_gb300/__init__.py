@@ -37,6 +37,8 @@ def _check_device(t: torch.Tensor, name: str):
 
 def _stream(device: torch.device) -> int:
     """The current stream of a CUDA device as an integer handle."""
+    if device.type != "cuda":
+        raise ValueError("expected a CUDA tensor, got one on %s" % device)
     index = device.index
     return torch._C._cuda_getCurrentRawStream(
         torch.cuda.current_device() if index is None else index)

@@ -24,3 +24,35 @@ def test_w_without_n(W, ok):
         assert (n > 0) == ok
         if W and ok:
             assert n == size(2, 3, at, (32, W, 0, 0))
+
+
+def _plan():
+    plan = P.SosFilter.__new__(P.SosFilter)  # its constructor needs a GPU
+    plan.n_channels, plan.kmax, plan.total = 1, 1, 64
+    plan.lengths_host = plan.lengths = torch.tensor([64])
+    plan.tuning, plan.ws_bytes = (0, 0, 0, 0), 1 << 20
+    plan.workspace = torch.zeros(16, dtype=torch.uint8)
+    plan.device = torch.device("cuda", 0)
+    plan._all = torch.ones(1, dtype=torch.int32)
+    plan._bws, plan._bws_bytes = plan.workspace, plan.ws_bytes
+    return plan
+
+
+@pytest.mark.parametrize("call", ["apply", "apply_part", "apply_baseline", "backward"])
+def test_host_tensors_never_reach_the_library(monkeypatch, call):
+    """The library takes device pointers: a call on CPU tensors is refused."""
+    for name in ("sos_apply", "sos_apply_part", "sos_apply_baseline", "sos_filter_backward"):
+        monkeypatch.setattr(_abi, name, lambda *a: pytest.fail("host pointer handed on"))
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda i: 0, raising=False)
+    plan, x, y = _plan(), torch.zeros(64), torch.zeros(64)
+    sos = torch.tensor([[[1.0, 0, 0, 1, 0, 0]]], dtype=torch.float64)
+    with pytest.raises(ValueError):
+        if call == "apply":
+            plan.apply(x, y)
+        elif call == "apply_part":
+            plan.apply_part("pipeline", x, y)
+        elif call == "apply_baseline":
+            plan.apply_baseline("scalar", x, y, 64)
+        else:
+            plan.backward(x, sos, plan._all, None, y, None)
