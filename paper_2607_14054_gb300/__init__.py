@@ -16,6 +16,7 @@ from __future__ import annotations
 
 from typing import Optional, Sequence
 
+import numpy as np
 import torch
 
 from . import _abi
@@ -44,12 +45,13 @@ def _stream(device: torch.device) -> int:
         torch.cuda.current_device() if index is None else index)
 
 
+_INTEGERS = {int, np.int64, np.int32}
+
+
 def _lengths(lengths) -> tuple:
-    if type(lengths) in (list, tuple):
-        try:
-            return tuple(map(int, lengths))
-        except (TypeError, ValueError):
-            pass  # nested, or tensors of several values
+    # plain integers, the usual case, need no tensor
+    if type(lengths) in (list, tuple) and set(map(type, lengths)) <= _INTEGERS:
+        return tuple(map(int, lengths))
     return tuple(int(v) for v in torch.as_tensor(lengths).reshape(-1).tolist())
 
 

@@ -133,7 +133,7 @@ def _tuning(t):
         return None
     if isinstance(t, sos_tuning):
         return ctypes.byref(t)
-    n, w, a, f = t if len(t) == 4 else (list(t) + [0, 0, 0, 0])[:4]
+    n, w, a, f = (*t, 0, 0, 0, 0)[:4]
     return _tuning_ref(int(n), int(w), int(a), int(f))
 
 

@@ -56,3 +56,22 @@ def test_host_tensors_never_reach_the_library(monkeypatch, call):
             plan.apply_baseline("scalar", x, y, 64)
         else:
             plan.backward(x, sos, plan._all, None, y, None)
+
+
+def test_lengths_as_torch_takes_them():
+    """A list of lengths means what torch.as_tensor makes of it, whatever its items."""
+    for v in ([5, 7], (5, 7), [[5, 7]], np.array([5, 7]), torch.tensor([5, 7]), [5.0, 7.9],
+              [torch.tensor(5), 7], [True, 7]):
+        assert P._lengths(v) == tuple(int(i) for i in torch.as_tensor(v).reshape(-1).tolist())
+    # beyond FP32's whole numbers
+    assert P._lengths([16_777_217.0]) == (16_777_216,)
+    with pytest.raises((TypeError, ValueError)):
+        P._lengths(["5"])
+
+
+def test_tuning_from_any_iterable():
+    lh = np.array([5000], dtype=np.int64)
+    n = _abi.sos_workspace_size(1, 3, lh.ctypes.data, (16, 8, 0, 0))
+    assert n > 0
+    for t in ([16, 8], (16, 8, 0), iter([16, 8, 0, 0]), (16, 8, 0, 0, 9)):
+        assert _abi.sos_workspace_size(1, 3, lh.ctypes.data, t) == n
