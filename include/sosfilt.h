@@ -37,6 +37,7 @@
  *   which are exactly the two scalar corrections the paper adds to the first
  *   element of the first two blocks (Sec. V-A, Eq. feedforward_block_uniform).
  *   zf rows k >= K[c] are written as zero; a zero-length channel returns zi.
+ *   zf may be zi's own buffer (a state updated in place; sos_stream wants two).
  * - Errors in arguments are detected on the host and returned before any
  *   work is enqueued.  Errors found on the device (nonzero a0 violated,
  *   non-finite coefficients, an unstable section when the stability check is

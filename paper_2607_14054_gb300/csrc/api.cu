@@ -16,6 +16,7 @@ int warpseg_ctas_per_sm(int N, int algo);
 int warpseg_warps_per_cta();
 cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32_t maxseg,
                           int32_t foreign, cudaStream_t stream);
+cudaError_t launch_save_state(Params& p, bool pipe, bool carry, cudaStream_t stream);
 cudaError_t launch_compare(const Params& p, int algo, int64_t seg_len, int64_t max_segs,
                            cudaStream_t stream);
 }  // namespace sosf
@@ -195,6 +196,7 @@ sos_status setup(int32_t n_channels, int32_t kmax, const int64_t* lengths_host, 
     p->W = tu.W;
     p->flags_opt = tu.flags;
     p->algo = tu.algo;
+    p->zstep = 2;
     const bool warp_segs = (tu.flags & SOS_FLAG_SECTION_PIPELINE) == 0;
     p->seg = segment_length(total_len, warp_segs ? ext_n(tu.N) : tu.N, tu.algo, tu.flags, warp_segs);
     {
@@ -252,6 +254,16 @@ sos_status check_signals(const float* x, const float* y, int64_t total) {
     return SOS_OK;
 }
 
+// whether the initial and the final states share memory: the states are then
+// set aside before any kernel writes one
+bool states_overlap(const Params& p) {
+    if (!p.zi || !p.zf) return false;
+    const char* a = reinterpret_cast<const char*>(p.zi);
+    const char* b = reinterpret_cast<const char*>(p.zf);
+    const size_t bytes = sizeof(float) * 2 * (size_t)p.kmax * (size_t)p.C;
+    return a < b + bytes && b < a + bytes;
+}
+
 // the launches of one pass over a call that setup() has filled p for
 sos_status enqueue_apply(Params p, int64_t tiles, const float* x, const float* zi, float* y,
                          float* zf, void* stream, int parts, bool reversed) {
@@ -267,6 +279,10 @@ sos_status enqueue_apply(Params p, int64_t tiles, const float* x, const float* z
     // sections: at least one CTA), launched early so that it starts without a
     // launch gap once the first has completed
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (states_overlap(p) &&
+        launch_save_state(p, (parts & kPartPipe) != 0, (parts & kPartCarry) != 0, st) !=
+            cudaSuccess)
+        return SOS_ERR_CUDA;
     bool early = false;
     if (total > 0 && (parts & kPartPipe)) {
         const int64_t sms = device_sms() > 0 ? device_sms() : 1;
@@ -367,17 +383,12 @@ sos_status sos_stream(const float* x, float* y, const float* zi, float* zf, int3
         const size_t bytes = sizeof(float) * (size_t)total;
         if (xb < yb + bytes && yb < xb + bytes) return SOS_ERR_ARG;
     }
-    if (zi && zf) {
-        // different warps of one channel read zi and write zf
-        const char* a = reinterpret_cast<const char*>(zi);
-        const char* b = reinterpret_cast<const char*>(zf);
-        const size_t bytes = sizeof(float) * 2 * (size_t)kmax * (size_t)n_channels;
-        if (a < b + bytes && b < a + bytes) return SOS_ERR_ARG;
-    }
     p.x = x;
     p.y = y;
     p.zi = zi;
     p.zf = zf;
+    // different warps of one channel read zi and write zf
+    if (states_overlap(p)) return SOS_ERR_ARG;
     if (chunk == 0) return SOS_OK;
     // segments: enough for every resident warp of the device to take one
     // when the channels alone do not fill it; each channel's own memory
@@ -427,6 +438,9 @@ sos_status sos_apply_baseline(int32_t algorithm, const float* x, int32_t n_chann
     p.y = y;
     p.zi = zi;
     p.zf = zf;
+    if (states_overlap(p) &&
+        launch_save_state(p, true, true, static_cast<cudaStream_t>(stream)) != cudaSuccess)
+        return SOS_ERR_CUDA;
     if (launch_compare(p, algorithm, seg_len, max_segs, static_cast<cudaStream_t>(stream)) !=
         cudaSuccess)
         return SOS_ERR_CUDA;

@@ -73,8 +73,8 @@ __global__ void sos_scalar_kernel(Params p, int64_t seg_len) {
             b2[k] = br.z;
             a1[k] = ab.x;
             a2[k] = ab.y;
-            z1[k] = g.first && p.zi ? p.zi[((int64_t)c * p.kmax + k) * 2 + 0] : 0.f;
-            z2[k] = g.first && p.zi ? p.zi[((int64_t)c * p.kmax + k) * 2 + 1] : 0.f;
+            z1[k] = g.first && p.zi ? p.zi[((int64_t)c * p.kmax + k) * p.zstep + 0] : 0.f;
+            z2[k] = g.first && p.zi ? p.zi[((int64_t)c * p.kmax + k) * p.zstep + 1] : 0.f;
         } else {
             b0[k] = 1.f;
             b1[k] = b2[k] = a1[k] = a2[k] = z1[k] = z2[k] = 0.f;
@@ -168,8 +168,8 @@ __global__ void __launch_bounds__(kBlkWarps * 32) sos_block_kernel(Params p, int
         px2[k] = px1[k] = py2[k] = py1[k] = 0.f;
         zi1[k] = zi2[k] = 0.f;
         if (k < g.K && g.first && p.zi) {
-            zi1[k] = p.zi[((int64_t)c * p.kmax + k) * 2 + 0];
-            zi2[k] = p.zi[((int64_t)c * p.kmax + k) * 2 + 1];
+            zi1[k] = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 0];
+            zi2[k] = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 1];
         }
     }
     const float* x = p.x + g.off;

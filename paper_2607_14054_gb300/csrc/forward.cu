@@ -168,8 +168,8 @@ __device__ __forceinline__ void data_section(const Params& p, float (&v)[N], int
     float zt1 = 0.f, zt2 = 0.f;
     if (CHAIN && warp == 0 && ti == 0 && p.zi) {
         const float gi = cf->misc.z;
-        zt1 = p.zi[((int64_t)c * p.kmax + k) * 2 + 0] * gi;
-        zt2 = p.zi[((int64_t)c * p.kmax + k) * 2 + 1] * gi;
+        zt1 = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 0] * gi;
+        zt2 = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 1] * gi;
     }
 
     // the section input at the channel's last sample (S8): the owning lane
@@ -310,8 +310,8 @@ __device__ __forceinline__ void coord_section(const Params& p, int k, int c, int
     const dfm2 Th = load_theta(cd, 1);
     float zi1 = 0.f, zi2 = 0.f;
     if (ti == 0 && p.zi) {
-        zi1 = p.zi[((int64_t)c * p.kmax + k) * 2 + 0];
-        zi2 = p.zi[((int64_t)c * p.kmax + k) * 2 + 1];
+        zi1 = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 0];
+        zi2 = p.zi[((int64_t)c * p.kmax + k) * p.zstep + 1];
     }
     __syncthreads();  // B1
     float A1 = 0.f, A2 = 0.f;
@@ -407,8 +407,8 @@ __global__ void __launch_bounds__((W + 1) * 32, MINB) sos_forward_kernel(Params 
             const int c = (int)(i / p.kmax), k = (int)(i % p.kmax);
             const ChanInfo ci = p.chan[c];
             if (k >= ci.K || ci.len == 0) {
-                const float z0 = (k < ci.K && p.zi) ? p.zi[i * 2 + 0] : 0.f;
-                const float z1 = (k < ci.K && p.zi) ? p.zi[i * 2 + 1] : 0.f;
+                const float z0 = (k < ci.K && p.zi) ? p.zi[i * p.zstep + 0] : 0.f;
+                const float z1 = (k < ci.K && p.zi) ? p.zi[i * p.zstep + 1] : 0.f;
                 p.zf[i * 2 + 0] = z0;
                 p.zf[i * 2 + 1] = z1;
             }
@@ -563,9 +563,30 @@ __global__ void __launch_bounds__((W + 1) * 32, MINB) sos_forward_kernel(Params 
     }
 }
 
+// The initial states of a call whose final states go to the same buffer, set
+// aside in its coefficient tables (Coef32::cpl): several warps read a channel's
+// state, and which of them is the first to write it is not known.  pipe, carry:
+// whether the channels within their horizon, and the others, are the call's.
+__global__ void save_state_kernel(Params p, bool pipe, bool carry) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)p.C * p.kmax) return;
+    const ChanInfo& ci = p.chan[i / p.kmax];
+    if (ci.horizon >= 0 && ci.len > 0 ? !pipe : !carry) return;
+    p.c32[i].cpl.z = p.zi[2 * i];
+    p.c32[i].cpl.w = p.zi[2 * i + 1];
+}
+
 // ---------------------------------------------------------------------------
 // launch
 // ---------------------------------------------------------------------------
+
+cudaError_t launch_save_state(Params& p, bool pipe, bool carry, cudaStream_t stream) {
+    const int64_t n = (int64_t)p.C * p.kmax;
+    save_state_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(p, pipe, carry);
+    p.zi = &p.c32[0].cpl.z;
+    p.zstep = sizeof(Coef32) / sizeof(float);
+    return cudaGetLastError();
+}
 
 struct KernelEntry {
     int N, W;

@@ -47,8 +47,8 @@ __device__ __forceinline__ void pipe_segment_section(const Params& p, const SegG
     float Z1 = 0.f, Z2 = 0.f;
     if (sg.cstart == 0 && p.zi) {
         const float gi = FACT ? misc.z : 1.f;
-        Z1 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 0] * gi;
-        Z2 = p.zi[((int64_t)sg.c * p.kmax + k) * 2 + 1] * gi;
+        Z1 = p.zi[((int64_t)sg.c * p.kmax + k) * p.zstep + 0] * gi;
+        Z2 = p.zi[((int64_t)sg.c * p.kmax + k) * p.zstep + 1] * gi;
     }
     const bool last_k = k == sg.K - 1;
     // the group holding the channel's last sample (zf), if in this segment

@@ -146,7 +146,8 @@ struct __align__(16) Coef32 {
     // or [[c, w], [w, c]] (real ones), c = -a1/2; w is at least 1 - r, r the larger
     // pole radius, so that coincident poles have a basis too
     float4 phi_c[7];
-    float4 cpl;           // w, 1/w
+    float4 cpl;           // w, 1/w; the section's initial state of a call with zi and zf in
+                          // one buffer (save_state_kernel)
     float4 phi_pow[5];    // Phi^(2^j), j = 0..4 (lane scan), DF2T basis
     float4 psi_pow[4];    // Psi^(2^r), r = 0..3 (warp scan)
     float4 psi_w[16];     // Psi^w, w = 0..15 (fold the tile state into warp w)
@@ -311,6 +312,8 @@ struct Params {
     float* gzi;          // backward: dL/dzi [C][kmax][2], or null
     double* gacc;        // backward: [C][kmax][5] sums for b0, b1, b2, a1, a2
     int64_t total;       // samples of all channels
+    int64_t zstep;       // floats from one section's zi to the next's: 2, the caller's layout, or
+                         // that of the copies in Coef32::cpl
     int64_t rev;         // 1: each channel's output is written time-reversed (sos_filtfilt)
 };
 

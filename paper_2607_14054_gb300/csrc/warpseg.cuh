@@ -389,8 +389,8 @@ __device__ __forceinline__ void ws_segment(const Params& p, volatile WsSeg& sg, 
         float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
         if (sg.first && p.zi) {
             const float gi = FACT ? __ldg(&p.c32[(int64_t)c * p.kmax + lane].misc.z) : 1.f;
-            z.x = __ldg(p.zi + ((int64_t)c * p.kmax + lane) * 2 + 0) * gi;
-            z.z = __ldg(p.zi + ((int64_t)c * p.kmax + lane) * 2 + 1) * gi;
+            z.x = __ldg(p.zi + ((int64_t)c * p.kmax + lane) * p.zstep + 0) * gi;
+            z.z = __ldg(p.zi + ((int64_t)c * p.kmax + lane) * p.zstep + 1) * gi;
         }
         zs[lane] = z;
     }
@@ -632,8 +632,8 @@ __device__ __forceinline__ void ws_long_phase(const Params& p, int lane) {
                 float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (sg.cstart == 0 && p.zi) {
                     const float gi = ci.mode != 0 && ci.ext < 3 ? cf0[lane].misc.z : 1.f;
-                    z.x = p.zi[((int64_t)sg.c * p.kmax + lane) * 2 + 0] * gi;
-                    z.z = p.zi[((int64_t)sg.c * p.kmax + lane) * 2 + 1] * gi;
+                    z.x = p.zi[((int64_t)sg.c * p.kmax + lane) * p.zstep + 0] * gi;
+                    z.z = p.zi[((int64_t)sg.c * p.kmax + lane) * p.zstep + 1] * gi;
                 }
                 zs[lane] = z;
             }
