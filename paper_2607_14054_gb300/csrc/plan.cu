@@ -505,6 +505,76 @@ __device__ float handoff_error(const double (*rows)[5], const float (*rowsf)[5],
     return 0x1p-24f * fmaxf(amp, 1.f);
 }
 
+// log ||h||_2 of the response of the normalised numerators, from below: the
+// energy of H on 32 points across a pole's peak, from two of its distances to
+// the circle below its angle to two above, the largest over the poles (those up
+// to four times as far from the circle as the nearest, equal ones once), by |1 -
+// p e^{-jw}|^2 = (1 - r)^2 + 4 r sin^2((w - phi) / 2), which does not cancel
+// next to the circle.  A response that builds up over many more than the 32
+// samples of horizon_norm is seen in full.  In logs: gains next to the circle
+// leave FP32's range.  One warp.
+__device__ float response_log_norm(const double (*rows)[5], const float (*rowsf)[5], int K,
+                                   int lane) {
+    const int np = 2 * K;
+    float r = 0.f, d = 1.f, phi = 0.f;  // lane i < 2K: pole i, its angle in half turns
+    if (lane < np) {
+        const double a1 = rows[lane >> 1][3], a2 = rows[lane >> 1][4];
+        const double disc = a1 * a1 - 4.0 * a2;
+        if (disc < 0.0) {
+            const double rd = sqrt(a2);
+            r = (float)rd;
+            d = (float)(1.0 - rd);
+            phi = 0.31830989f * atan2f(sqrtf((float)-disc), (float)-a1);
+            if (lane & 1) phi = -phi;
+        } else {
+            const double z = 0.5 * ((lane & 1) ? -a1 - sqrt(disc) : -a1 + sqrt(disc));
+            r = (float)fabs(z);
+            d = (float)(1.0 - fabs(z));
+            phi = z < 0.0 ? 1.f : 0.f;
+        }
+    }
+    float best = -INFINITY, near = d;
+    for (int o = 16; o > 0; o >>= 1) near = fminf(near, __shfl_xor_sync(0xffffffffu, near, o));
+    const unsigned same = __match_any_sync(0xffffffffu, (unsigned long long)__float_as_uint(d) << 32 |
+                                                            __float_as_uint(phi));
+    // lanes of poles to try: not a conjugate, not a copy of a lower lane's
+    unsigned todo = __ballot_sync(0xffffffffu, lane < np && phi >= 0.f && d <= 4.f * near &&
+                                                   __ffs(same) - 1 == lane);
+    for (; todo; todo &= todo - 1u) {
+        const int j = __ffs(todo) - 1;
+        const float dj = __shfl_sync(0xffffffffu, d, j), pj = __shfl_sync(0xffffffffu, phi, j);
+        const float w = fmaf(0.31830989f * dj, 0.125f * (lane + 0.5f) - 2.f, pj);
+        const bool on = w >= 0.f && w <= 1.f;
+        float L = 0.f;
+        float a2 = 1.f;  // a section's two factors, above 1e-32
+        for (int i = 0; i < np; ++i) {
+            const float ri = __shfl_sync(0xffffffffu, r, i), di = __shfl_sync(0xffffffffu, d, i);
+            const float s = sinpif(0.5f * (w - __shfl_sync(0xffffffffu, phi, i)));
+            a2 *= fmaf(di, di, 4.f * ri * s * s);
+            if (i & 1) {
+                L -= __logf(fmaxf(a2, 1e-37f));
+                a2 = 1.f;
+            }
+        }
+        const float c1 = cospif(w), s1 = sinpif(w), c2 = fmaf(2.f * c1, c1, -1.f), s2 = 2.f * s1 * c1;
+        for (int k = 0; k < K; ++k) {
+            const float ims = 1.f / num_scale(rowsf[k]);
+            const float b0 = rowsf[k][0] * ims, b1 = rowsf[k][1] * ims, b2 = rowsf[k][2] * ims;
+            const float re = fmaf(b2, c2, fmaf(b1, c1, b0)), im = fmaf(b2, s2, b1 * s1);
+            L += __logf(fmaxf(fmaf(re, re, im * im), 1e-30f));
+        }
+        if (!on) L = -INFINITY;
+        float m = L;
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        float e = on ? __expf(L - m) : 0.f;
+        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        // (1 / pi) sum |H|^2 dw
+        const float t = 0.5f * (m + __logf(fmaxf(e, 1e-30f) * 0.125f * dj * 0.31830989f));
+        if (t < 1e30f) best = fmaxf(best, t);
+    }
+    return best;
+}
+
 // A memory horizon without partial fractions, for cascades whose poles
 // coincide (or nearly so) and so have none to use: with r the largest pole
 // modulus, each section's all-pole response is bounded by (n + 1) r^n and its
@@ -517,9 +587,22 @@ __device__ float handoff_error(const double (*rows)[5], const float (*rowsf)[5],
 // horizon, but it holds for repeated poles.  tz: the same for the response
 // of a unit initial state (it enters a section's recursion like an impulse
 // of at most unit size, so B_k is taken as at least 1).  -1 where r >= 1 or
-// no such P below 2^30.  One warp, the same result in every lane.
-__device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int lane, int& tz) {
+// no such P below 2^30.
+// h2 is that of the normalised numerators (num_scale), B_k is not: for small
+// numerators (a low cutoff) P is short by the log of their product over 1 - r,
+// and it was measured so: four equal sections lost up to 2e-3 of the output in
+// the tails they dropped.  What such a channel's segments are warmed up over is
+// therefore warm >= P, for which the tail's energy is below kFallbackEps ||h||_2,
+// both in true scale (response_log_norm, or h2 where that is larger), by the
+// same bound but for sections whose pole pair lies far enough from the axis for
+// r^n / sin(angle) to be less than (n + 1) r^n over P samples: their
+// coefficients are then those of one factor, not two.  For two equal sections it
+// comes to P again (4,464 for 4,416 samples at a cutoff of 0.002).
+// One warp, the same result in every lane.
+__device__ int horizon_fallback(const double (*rows)[5], const float (*rowsf)[5], int K, float h2,
+                                int lane, int& tz, int& warm) {
     tz = -1;
+    warm = -1;
     if (K < 1 || !(h2 > 0.f)) return -1;
     double r = 0.0, logA = 0.0, logAs = 0.0;
     for (int k = 0; k < K; ++k) {
@@ -541,20 +624,14 @@ __device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int la
     if (!(r < 1.0 - 1e-12)) return -1;
     if (r < 1e-300) {  // a finite response
         tz = ((2 * K + 1) + 15) / 16 * 16;
+        warm = tz;
         return tz;
     }
-    const double m = 2.0 * K, lr = log(r), lgm = lgamma(m);
-    const double target = log((double)kHorizonEps * (double)h2);
-    // the first n past the peak (ratio < 1) where the log tail bound with
-    // prefactor log a is below the target, in multiples of 16; -1 if none
-    auto first = [&](double loga) -> int {
-        // (n + m - 1)! / n! = (n + 1) .. (n + m - 1): at most 15 factors below 2^31
-        auto tail = [&](double n) {
-            const double ratio = r * (n + m) / (n + 1.0);
-            double pr = 1.0;
-            for (int i = 1; i < 2 * K; ++i) pr *= n + i;
-            return loga + log(pr) - lgm + n * lr - log1p(-ratio);
-        };
+    const double lr = log(r);
+    // the first n past the peak of m factors' terms (ratio < 1) where tail(n, the
+    // ratio) is below the target, in multiples of 16; -1 if none
+    auto first = [&](double m, double target, auto tail_at) -> int {
+        auto tail = [&](double n) { return tail_at(n, r * (n + m) / (n + 1.0)); };
         double lo = fmax(ceil((m * r - 1.0) / (1.0 - r)) + 1.0, m);
         double hi = 1073741824.0;
         // (the same in every lane) hi satisfies the bound, lo does not; the
@@ -577,10 +654,46 @@ __device__ int horizon_fallback(const double (*rows)[5], int K, float h2, int la
         const int64_t n = ((int64_t)hi + 15) / 16 * 16;
         return n < (int64_t)1 << 30 ? (int)n : -1;
     };
-    const int P = first(logA - 2.0 * K * lr);
+    const double m = 2.0 * K, lgm = lgamma(m);
+    const double target = log((double)kHorizonEps * (double)h2);
+    // the log of the tail's sum with prefactor log a
+    auto sum_tail = [&](double loga) {
+        return [=](double n, double ratio) {
+            // (n + m - 1)! / n! = (n + 1) .. (n + m - 1): at most 15 factors below 2^31
+            double pr = 1.0;
+            for (int i = 1; i < 2 * K; ++i) pr *= n + i;
+            return loga + log(pr) - lgm + n * lr - log1p(-ratio);
+        };
+    };
+    const int P = first(m, target, sum_tail(logA - 2.0 * K * lr));
     if (P < 0) return -1;
-    tz = first(logAs - 2.0 * K * lr);
-    return tz < 0 ? -1 : P;
+    tz = first(m, target, sum_tail(logAs - 2.0 * K * lr));
+    if (tz < 0) return -1;
+    // the warm-up (logs in FP32: its bound is not that sharp)
+    float logC = 0.f, logm = 0.f, lgc = 0.f;
+    int mc = 0;
+    for (int k = 0; k < K; ++k) {
+        const double a1 = rows[k][3], a2 = rows[k][4];
+        const float im = sqrtf(fmaxf((float)(4.0 * a2 - a1 * a1), 0.f));  // 2 Im p
+        const float csc = im > 0.f ? 2.f * sqrtf((float)a2) / im : INFINITY;
+        if (csc * (float)(2 * K) < (float)P) {
+            logC += __logf(csc);
+            mc += 1;
+        } else {
+            mc += 2;
+        }
+        logm += __logf(num_scale(rowsf[k]));
+    }
+    for (int i = 2; i < mc; ++i) lgc += __logf((float)i);
+    const float lh = fmaxf(response_log_norm(rows, rowsf, K, lane), __logf(h2)) + logm;
+    const double loga = logA - 2.0 * K * lr + (double)(logC - lgc);
+    const int Pw = first(mc, (double)(lh + __logf(kFallbackEps)), [=](double n, double ratio) {
+        float t = 0.f;
+        for (int i = 1; i < mc; ++i) t += __logf((float)(n + i));
+        return loga + n * lr + (double)(t - 0.5f * __logf((float)(1.0 - ratio * ratio)));
+    });
+    warm = Pw > P ? Pw : P;
+    return P;
 }
 
 // The horizon from the per-pole terms and ||h||_2 >= h2 (the pole warp), and
@@ -919,18 +1032,20 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         // both sides), and in forward plans where the channel is long enough
         // for at least eight segments (the look-back is faster below that)
         if (P < 0 && !carry_only && Kc > 0) {
-            int Pf = -1, tzf = -1;
-            Pf = horizon_fallback(s_row, Kc, s_h2, lane, tzf);
-            const int64_t want = Pf >= 0 ? (2LL * Pf > tzf ? 2LL * Pf : (int64_t)tzf) : 0;
+            int Pf = -1, tzf = -1, warm = -1;
+            Pf = horizon_fallback(s_row, s_rowf, Kc, s_h2, lane, tzf, warm);
+            int64_t want = Pf >= 0 ? (2LL * Pf > tzf ? 2LL * Pf : (int64_t)tzf) : 0;
             const int64_t lenc = p.lengths[c];
             if (Pf >= 0 && ((p.flags_opt & kFlagBackwardPlan) || lenc >= 8 * want)) {
                 const int64_t G = 32LL * p.N;
-                P = Pf;
+                P = warm;
+                tzf = tzf > warm ? tzf : warm;
+                want = 2LL * P > tzf ? 2LL * P : (int64_t)tzf;
                 seg = p.seg;
                 const int64_t GT = 32LL * ext_n(p.N);
                 if (want > seg) seg = (want + GT - 1) / GT * GT;
-                zdecay = tzf > Pf ? tzf : Pf;
-                minseg = (int32_t)((Pf + G - 1) / G * G > G ? (Pf + G - 1) / G * G : G);
+                zdecay = tzf;
+                minseg = (int32_t)((P + G - 1) / G * G > G ? (P + G - 1) / G * G : G);
                 minseg_z = (int32_t)((tzf + G - 1) / G * G > minseg ? (tzf + G - 1) / G * G
                                                                      : minseg);
             }

@@ -107,6 +107,10 @@ static_assert(sizeof(ChanInfo) == 80, "channel table entry");
 // far below FP32 rounding.  Longer memories (P > T / 2, poles on or near the
 // unit circle, coincident poles) keep the decoupled look-back.
 constexpr float kHorizonEps = 0x1p-30f;
+// Coincident poles' warm-up (horizon_fallback): the energy of the response's
+// dropped tail relative to ||h||_2.  What a segment drops it drops over its first
+// 1 / (1 - r) samples, a few per cent of it: below FP32's rounding of the output.
+constexpr float kFallbackEps = 0x1p-22f;
 
 // Channels with a longer horizon keep the scalar order of operations of
 // long_section.cuh on the warp-segment kernel (there the reason), in segments
