@@ -29,22 +29,33 @@ constexpr int32_t kAbiVersion = 1;
 
 struct Tune {
     int N, W, algo, flags;
+    int Nc, Wc;  // the look-back kernel's
 };
 
 // The library's defaults: N = 64, W = 4 (tiles of 8,192 samples).  N given alone
 // takes W = 8, W given alone N = 32, for which every documented W is compiled.
 bool resolve_tuning(const sos_tuning* t, Tune* out) {
-    Tune r{64, 4, 1, 0};
+    Tune r{64, 4, 1, 0, 0, 0};
+    bool chosen = false;
     if (t) {
         if (t->n_blocks || t->warps) {
             r.N = t->n_blocks ? t->n_blocks : 32;
             r.W = t->warps ? t->warps : 8;
+            chosen = true;
         }
         if (t->algo) r.algo = t->algo;
         r.flags = t->flags;
     }
     if (r.algo != 1 && r.algo != 2) return false;
-    if (!forward_supported(r.N, r.W) || !pipe_supported(r.N)) return false;
+    // Carried channels keep N = 32, W = 8 (the same tiles) where the call leaves
+    // both to the library: eight data warps a CTA for four, and runs of 32
+    // samples for 64, whose errors are a third larger (crossovers of cutoff
+    // 0.0015..0.05).  us at (32, 8) and (64, 4), carried throughout: 2^24 samples,
+    // K = 8, 376..386 and 360..386; K = 2, 148 and 158; 1024 of 4000, K = 3, 41 and 46; 4096
+    // of 1000, K = 8, 206 and 247; 2^20, K = 8, 45 and 44.
+    r.Nc = chosen ? r.N : 32;
+    r.Wc = chosen ? r.W : 8;
+    if (!forward_supported(r.Nc, r.Wc) || !pipe_supported(r.N)) return false;
     *out = r;
     return true;
 }
@@ -194,6 +205,8 @@ sos_status setup(int32_t n_channels, int32_t kmax, const int64_t* lengths_host, 
     p->kmax = kmax;
     p->N = tu.N;
     p->W = tu.W;
+    p->Nc = tu.Nc;
+    p->Wc = tu.Wc;
     p->flags_opt = tu.flags;
     p->algo = tu.algo;
     p->zstep = 2;

@@ -615,7 +615,7 @@ cudaError_t launch_forward(const Params& p, int64_t host_tiles, cudaStream_t str
                            bool early) {
     const KernelEntry* ke = nullptr;
     for (const auto& e : kEntries)
-        if (e.N == p.N && e.W == p.W) ke = &e;
+        if (e.N == p.Nc && e.W == p.Wc) ke = &e;
     if (!ke) return cudaErrorInvalidValue;
     int dev = 0;
     cudaError_t err = cudaGetDevice(&dev);
@@ -633,14 +633,14 @@ cudaError_t launch_forward(const Params& p, int64_t host_tiles, cudaStream_t str
                                    (int)ke->smem);
         if (err != cudaSuccess) return err;
         int occ = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ke->fn, (p.W + 1) * 32, ke->smem);
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ke->fn, (p.Wc + 1) * 32, ke->smem);
         if (err != cudaSuccess) return err;
         s_occ[dev][idx] = occ > 0 ? occ : 1;
     }
     int64_t grid = (int64_t)s_sms[dev] * s_occ[dev][idx];
     if (host_tiles < grid) grid = host_tiles;
     if (grid < 1) return cudaSuccess;
-    return launch_params(ke->fn, grid, (p.W + 1) * 32, ke->smem, p, stream, early);
+    return launch_params(ke->fn, grid, (p.Wc + 1) * 32, ke->smem, p, stream, early);
 }
 
 }  // namespace sosf

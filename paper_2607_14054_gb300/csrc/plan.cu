@@ -843,6 +843,10 @@ __device__ __forceinline__ int32_t key_fair(const Params& p) {
     return p.fair < 0x7fffffff ? (int32_t)p.fair : 0x7fffffff;
 }
 
+// W and the look-back's in the key: explicit and default tunings that agree in N
+// and W may differ in how a carried channel's tables are built
+__device__ __forceinline__ int32_t key_warps(const Params& p) { return p.W | p.Wc << 8; }
+
 // Block c < C: the coefficient tables and the memory horizon of channel c.
 // Returns false when the channel's tables were kept from the previous plan on
 // this workspace (plan cache: same raw sos rows bit for bit, same K and
@@ -918,7 +922,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         const int32_t kv = kh->valid, kK = kh->K;
         const int64_t kl = kh->len, len = p.lengths[c];
         const bool same = !(p.flags_opt & SOS_FLAG_REPLAN) & (hv == 1) & (hN == p.N) &
-                          (hW == p.W) & (ha == p.algo) & (hf == p.flags_opt) & (hk == kmax) &
+                          (hW == key_warps(p)) & (ha == p.algo) & (hf == p.flags_opt) & (hk == kmax) &
                           (hC == p.C) & (hs == p.seg) & (hfair == key_fair(p)) & (hc == p.cap_tiles) & (kv == 1) &
                           (kK == K) & (kl == len);
         s_same[kMaxSections] = same;
@@ -1103,7 +1107,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
     if (!active) return true;
 
     // ---- Phi: double-float squaring chain (lane 0) ----
-    const int N = p.N, W = p.W;
+    const int N = p.N;
     if (lane == 0) {
         const dfm2 A{df_of_double(-a1), df{1.f, 0.f}, df_of_double(-a2), df{0.f, 0.f}};
         dfm2 P = A;
@@ -1245,11 +1249,12 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
             !(p.flags_opt & (kFlagBackwardPlan | SOS_FLAG_SECTION_PIPELINE)))
             if (!is_long(p, s_horizon)) warp_segments(p, c, p.lengths[c], s_horizon, e);
     }
+    // the powers for n = N or N/2 samples per lane, the j-th squaring from there
+    auto pow2_of = [&](int n, int j) {
+        return n == N ? s_chain[k][j] : j == 0 ? s_part[k][0] : s_chain[k][j - 1];
+    };
     if (s_horizon >= 0) {
-        // the powers for ext_n(N) samples per lane, the j-th squaring from there
-        auto pow2 = [&](int j) {
-            return ext_n(N) == N ? s_chain[k][j] : j == 0 ? s_part[k][0] : s_chain[k][j - 1];
-        };
+        auto pow2 = [&](int j) { return pow2_of(ext_n(N), j); };
         if (is_long(p, s_horizon)) {
             // a long-memory channel: the DF2T powers with their low parts
             dfm2 P = dfm_identity();
@@ -1276,8 +1281,17 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         }
         return true;
     }
+    const int Nc = p.Nc;
+    if (Nc != N) {
+        dfm2 P = dfm_identity();
+        for (int j = 0; j < 5; ++j)
+            if ((lane >> j) & 1) P = dfm_mul(P, pow2_of(Nc, j));
+        out32->lane_pow[lane] = to_f4(P);
+        if (lane < 5) out32->phi_pow[lane] = to_f4(pow2_of(Nc, lane));
+    }
     if (lane == 0) {
-        dfm2 P = dfm_mul(s_chain[k][4], s_chain[k][4]);  // Psi = Phi^32
+        // Psi = Phi^32 (s_chain[k][4] is it for Nc = N/2)
+        dfm2 P = Nc == N ? dfm_mul(s_chain[k][4], s_chain[k][4]) : s_chain[k][4];
         s_chain[k][5] = P;
         for (int r = 1; r < 5; ++r) {
             P = dfm_mul(P, P);
@@ -1293,9 +1307,9 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
     }
     if (lane < 4) out32->psi_pow[lane] = to_f4(s_chain[k][5 + lane]);
     if (lane == 0) {
-        dfm2 Th = dfm_identity();  // Theta = Psi^W, any W <= 31
+        dfm2 Th = dfm_identity();  // Theta = Psi^Wc, any Wc <= 31
         for (int r = 0; r < 5; ++r)
-            if ((W >> r) & 1) Th = dfm_mul(Th, s_chain[k][5 + r]);
+            if ((p.Wc >> r) & 1) Th = dfm_mul(Th, s_chain[k][5 + r]);
         s_chain[k][10] = Th;
         for (int i = 1; i < 10; ++i) s_chain[k][10 + i] = dfm_mul(s_chain[k][9 + i], s_chain[k][9 + i]);
     }
@@ -1541,7 +1555,7 @@ __global__ void __launch_bounds__(kPlanThreads) plan_kernel(Params p) {
     if (threadIdx.x == 0) {
         WsHeader* h = p.hdr;
         h->key_N = p.N;
-        h->key_W = p.W;
+        h->key_W = key_warps(p);
         h->key_algo = p.algo;
         h->key_flags = p.flags_opt;
         h->key_kmax = p.kmax;

@@ -152,7 +152,9 @@ struct __align__(16) Coef32 {
     float4 phi_c[7];
     float4 cpl;           // w, 1/w; the section's initial state of a call with zi and zf in
                           // one buffer (save_state_kernel)
-    float4 phi_pow[5];    // Phi^(2^j), j = 0..4 (lane scan), DF2T basis
+    // DF2T basis; for a carried channel Phi = A^Nc and W = Wc (Params), for a
+    // long-memory one Phi = A^ext_n(N)
+    float4 phi_pow[5];    // Phi^(2^j), j = 0..4 (lane scan)
     float4 psi_pow[4];    // Psi^(2^r), r = 0..3 (warp scan)
     float4 psi_w[16];     // Psi^w, w = 0..15 (fold the tile state into warp w)
     float4 lane_pow[32];  // Phi^l, l = 0..31 (fold the warp state into lane l)
@@ -301,8 +303,10 @@ struct Params {
     int32_t kmax;
     int32_t N;           // samples per lane
     int32_t W;           // warps per tile
+    int32_t Nc, Wc;      // the same of the look-back kernel (Nc Wc = N W)
     int32_t flags_opt;   // SOS_FLAG_*
     int32_t algo;        // recursive-stage solver: 1 PH, 2 CR where well conditioned
+    int32_t pad;
     int64_t seg;         // tile length of the channels within their horizon (samples, a
                          // multiple of 32 N): the segments of the section pipeline and
                          // the backward
