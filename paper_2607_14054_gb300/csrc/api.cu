@@ -12,7 +12,7 @@ cudaError_t launch_pipe(const Params& p, int64_t grid, cudaStream_t stream, bool
 bool forward_supported(int N, int W);
 bool pipe_supported(int N);
 cudaError_t launch_warpseg(const Params& p, int64_t grid, cudaStream_t stream, bool early);
-int warpseg_ctas_per_sm(int N, int algo);
+int warpseg_ctas_per_sm(int N, int algo, int dev);
 int warpseg_warps_per_cta();
 cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32_t maxseg,
                           int32_t foreign, cudaStream_t stream);
@@ -73,11 +73,10 @@ sos_tuning backward_tuning(const sos_tuning* t) {
     return r;
 }
 
-// SMs of the current device (cached per device); 0 if unknown.
-int device_sms() {
-    static int s_sms[64] = {0};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+// SMs of the current device, whose slot is dev (cached); 0 if unknown.
+int device_sms(int dev) {
+    static int s_sms[kDeviceSlots] = {};
+    if (dev < 0) return 0;
     if (s_sms[dev] == 0 &&
         cudaDeviceGetAttribute(&s_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
@@ -94,15 +93,14 @@ constexpr int kPipeCtasPerSm = 2;
 // of long-memory channels).
 // CTAs per SM of a warp-segment launch: the tuning's request (flag bits
 // 8..11), at most as many as fit; 0 = as many as fit.
-int warpseg_ctas(int N, int algo, int flags) {
-    const int fit = warpseg_ctas_per_sm(N, algo);
+int warpseg_ctas(int N, int algo, int flags, int dev) {
+    const int fit = warpseg_ctas_per_sm(N, algo, dev);
     const int req = (flags >> 8) & 15;
     return req > 0 && req < fit ? req : fit;
 }
 
-int64_t segment_length(int64_t total_len, int N, int algo, int flags, bool warp_segments) {
+int64_t segment_length(int64_t total_len, int N, int flags, bool warp_segments, int sms) {
     const int64_t group = 32LL * N;
-    const int sms = device_sms() > 0 ? device_sms() : 148;
     int64_t units = (int64_t)sms * kPipeCtasPerSm, gmin = 8;
     if (warp_segments) {
         const int req = (flags >> 8) & 15;
@@ -211,12 +209,13 @@ sos_status setup(int32_t n_channels, int32_t kmax, const int64_t* lengths_host, 
     p->algo = tu.algo;
     p->zstep = 2;
     const bool warp_segs = (tu.flags & SOS_FLAG_SECTION_PIPELINE) == 0;
-    p->seg = segment_length(total_len, warp_segs ? ext_n(tu.N) : tu.N, tu.algo, tu.flags, warp_segs);
+    p->dev = device_slot();
+    const int sms = device_sms(p->dev) > 0 ? device_sms(p->dev) : 148;
+    p->seg = segment_length(total_len, warp_segs ? ext_n(tu.N) : tu.N, tu.flags, warp_segs, sms);
     {
         const int64_t group = 32LL * tu.N;
-        const int64_t sms = device_sms() > 0 ? device_sms() : 148;
-        const int occ = warpseg_ctas(tu.N, tu.algo, tu.flags);
-        const int64_t warps = sms * (occ > 0 ? occ : 1) * warpseg_warps_per_cta();
+        const int occ = warpseg_ctas(tu.N, tu.algo, tu.flags, p->dev);
+        const int64_t warps = (int64_t)sms * (occ > 0 ? occ : 1) * warpseg_warps_per_cta();
         p->fair = (total_len + warps - 1) / warps;
         int64_t g = (p->fair + group - 1) / group;
         g = g < 1 ? 1 : g > 64 ? 64 : g;
@@ -298,7 +297,7 @@ sos_status enqueue_apply(Params p, int64_t tiles, const float* x, const float* z
         return SOS_ERR_CUDA;
     bool early = false;
     if (total > 0 && (parts & kPartPipe)) {
-        const int64_t sms = device_sms() > 0 ? device_sms() : 1;
+        const int64_t sms = device_sms(p.dev) > 0 ? device_sms(p.dev) : 1;
         cudaError_t e;
         // launched early (programmatic dependent launch): its CTAs become
         // resident while the preceding kernel (normally the plan) finishes,
@@ -306,7 +305,7 @@ sos_status enqueue_apply(Params p, int64_t tiles, const float* x, const float* z
         if (p.flags_opt & SOS_FLAG_SECTION_PIPELINE)
             e = launch_pipe(p, sms * kPipeCtasPerSm, st, true);
         else
-            e = launch_warpseg(p, sms * warpseg_ctas(p.N, p.algo, p.flags_opt), st, true);
+            e = launch_warpseg(p, sms * warpseg_ctas(p.N, p.algo, p.flags_opt, p.dev), st, true);
         if (e != cudaSuccess) return SOS_ERR_CUDA;
         early = true;
     }
@@ -407,8 +406,8 @@ sos_status sos_stream(const float* x, float* y, const float* zi, float* zf, int3
     // when the channels alone do not fill it; each channel's own memory
     // horizon may lengthen its segments on the device
     const int64_t group = 32LL * p.N;
-    const int sms = device_sms() > 0 ? device_sms() : 148;
-    const int occ = warpseg_ctas(p.N, 1, 0);
+    const int sms = device_sms(p.dev) > 0 ? device_sms(p.dev) : 148;
+    const int occ = warpseg_ctas(p.N, 1, 0, p.dev);
     const int64_t warps = (int64_t)sms * (occ > 0 ? occ : 1) * warpseg_warps_per_cta();
     int64_t per = warps / n_channels;
     if (per < 1) per = 1;
@@ -600,7 +599,7 @@ sos_status sos_plan_recomputed(void* workspace, int32_t* channels, void* stream)
 
 namespace sosf {
 cudaError_t launch_adjoint(const Params& p, int sms, double* grad_sos, cudaStream_t stream);
-int64_t adjoint_segments(int N, int sms);
+int64_t adjoint_segments(int N, int sms, int dev);
 int64_t adjoint_ck_slots(int N, int64_t total_len, int32_t C);
 }  // namespace sosf
 
@@ -631,10 +630,10 @@ BwdLayout bwd_layout(size_t base, int32_t C, int32_t kmax, int64_t total_len, in
 // partial segment does not start a second round on a few CTAs; a horizon
 // of up to half a segment fits.
 int64_t backward_segment_length(const int64_t* lengths_host, int32_t C, int64_t total_len,
-                                int N) {
+                                int N, int dev) {
     const int64_t group = 32LL * N;
-    const int sms = device_sms() > 0 ? device_sms() : 148;
-    int64_t units = adjoint_segments(N, sms);
+    const int sms = device_sms(dev) > 0 ? device_sms(dev) : 148;
+    int64_t units = adjoint_segments(N, sms, dev);
     if (units < 1) units = 1;
     int64_t g0 = (total_len + units * group - 1) / (units * group);
     if (g0 < 8) g0 = 8;
@@ -696,7 +695,7 @@ sos_status sos_filter_backward(const float* x, const double* sos, const int32_t*
     // the backward plan: no look-back (a channel without a memory horizon is
     // one segment), segments sized for the adjoint kernel's warps
     p.flags_opt |= kFlagBackwardPlan;
-    p.seg = backward_segment_length(lengths_host, n_channels, total, p.N);
+    p.seg = backward_segment_length(lengths_host, n_channels, total, p.N, p.dev);
     p.ck = reinterpret_cast<float*>(ws + BL.ck);
     p.gacc = reinterpret_cast<double*>(ws + BL.gacc);
     if (launch_plan(p, sm) != cudaSuccess) return SOS_ERR_CUDA;
@@ -711,7 +710,7 @@ sos_status sos_filter_backward(const float* x, const double* sos, const int32_t*
     p.gzf = grad_zf;
     p.gx = grad_x;
     p.gzi = grad_zi;
-    const int sms = device_sms() > 0 ? device_sms() : 1;
+    const int sms = device_sms(p.dev) > 0 ? device_sms(p.dev) : 1;
     if (launch_adjoint(p, sms, grad_sos, sm) != cudaSuccess) return SOS_ERR_CUDA;
     return SOS_OK;
 }

@@ -587,9 +587,8 @@ size_t adj_smem(int N) {
 }  // namespace
 
 // segments (CTAs) of the adjoint kernel resident on the device (0 on error)
-int64_t adjoint_segments(int N, int sms) {
+int64_t adjoint_segments(int N, int sms, int dev) {
     static int s_occ[kDeviceSlots][3] = {};
-    const int dev = device_slot();
     if (dev < 0) return 0;
     const int idx = N == 16 ? 0 : N == 32 ? 1 : 2;
     if (s_occ[dev][idx] == 0) {
@@ -612,7 +611,7 @@ int64_t adjoint_ck_slots(int N, int64_t total_len, int32_t C) {
 }
 
 cudaError_t launch_adjoint(const Params& p, int sms, double* grad_sos, cudaStream_t stream) {
-    const int64_t ctas = adjoint_segments(p.N, sms);
+    const int64_t ctas = adjoint_segments(p.N, sms, p.dev);
     if (ctas < 1) return cudaErrorInvalidConfiguration;
     if (p.total > 0) {
         const cudaError_t e = launch_params(adj_fn(p.N), ctas, kBwThreads,

@@ -251,7 +251,7 @@ cudaError_t launch_compare(const Params& p, int algo, int64_t seg_len, int64_t m
     } else {
         const size_t smem = sizeof(float) * kBlkWarps * kMaxSections * 64;
         static bool attr[kDeviceSlots] = {};
-        const int dev = device_slot();
+        const int dev = p.dev;
         if (dev < 0) return cudaErrorInvalidDevice;
         if (!attr[dev]) {
             const cudaError_t e = cudaFuncSetAttribute(

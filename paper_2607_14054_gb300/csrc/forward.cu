@@ -617,13 +617,12 @@ cudaError_t launch_forward(const Params& p, int64_t host_tiles, cudaStream_t str
     for (const auto& e : kEntries)
         if (e.N == p.Nc && e.W == p.Wc) ke = &e;
     if (!ke) return cudaErrorInvalidValue;
-    int dev = 0;
-    cudaError_t err = cudaGetDevice(&dev);
-    if (err != cudaSuccess) return err;
-    static int s_sms[64] = {0};
-    static int s_occ[64][16] = {{0}};
+    const int dev = p.dev;
+    if (dev < 0) return cudaErrorInvalidDevice;
+    cudaError_t err;
+    static int s_sms[kDeviceSlots] = {};
+    static int s_occ[kDeviceSlots][16] = {};
     const int idx = (int)(ke - kEntries);
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (s_sms[dev] == 0) {
         err = cudaDeviceGetAttribute(&s_sms[dev], cudaDevAttrMultiProcessorCount, dev);
         if (err != cudaSuccess) return err;

@@ -265,7 +265,7 @@ cudaError_t launch_pipe(const Params& p, int64_t grid, cudaStream_t stream, bool
                                                                 : SOSF_PIPE(64, false));
     const size_t smem = 2 * sizeof(float) * 32 * (size_t)(p.N + 4) * kPipeRing;
     static bool attr[kDeviceSlots][2][3] = {};
-    const int dev = device_slot();
+    const int dev = p.dev;
     if (dev < 0) return cudaErrorInvalidDevice;
     const int idx = p.N == 16 ? 0 : p.N == 32 ? 1 : 2;
     if (!attr[dev][z][idx]) {

@@ -1574,7 +1574,7 @@ cudaError_t launch_plan(const Params& p, cudaStream_t stream) {
     while (n < p.C && n < kMaxSortChannels) n <<= 1;
     const size_t smem = p.C <= kMaxSortChannels ? sizeof(unsigned long long) * (size_t)n : 0;
     static bool attr_set[kDeviceSlots] = {};
-    const int dev = device_slot();
+    const int dev = p.dev;
     if (dev < 0) return cudaErrorInvalidDevice;
     if (!attr_set[dev]) {
         const cudaError_t err =

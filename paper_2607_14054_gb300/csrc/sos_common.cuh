@@ -306,7 +306,7 @@ struct Params {
     int32_t Nc, Wc;      // the same of the look-back kernel (Nc Wc = N W)
     int32_t flags_opt;   // SOS_FLAG_*
     int32_t algo;        // recursive-stage solver: 1 PH, 2 CR where well conditioned
-    int32_t pad;
+    int32_t dev;         // host: the device's slot (device_slot), looked up once a call
     int64_t seg;         // tile length of the channels within their horizon (samples, a
                          // multiple of 32 N): the segments of the section pipeline and
                          // the backward

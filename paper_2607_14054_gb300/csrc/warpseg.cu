@@ -26,10 +26,9 @@ size_t ws_smem(int N) {
 }  // namespace
 
 // CTAs of the warp-segment kernel (algo 2: the cyclic-reduction one)
-// resident per SM of the current device (0 on error)
-int warpseg_ctas_per_sm(int N, int algo) {
+// resident per SM of the current device, whose slot is dev (0 on error)
+int warpseg_ctas_per_sm(int N, int algo, int dev) {
     static int s_occ[kDeviceSlots][2][3] = {};
-    const int dev = device_slot();
     if (dev < 0) return 0;
     const int idx = N == 16 ? 0 : N == 32 ? 1 : 2, a = algo == 2 ? 1 : 0;
     if (s_occ[dev][a][idx] == 0) {
@@ -56,7 +55,7 @@ cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32
                           int32_t foreign, cudaStream_t stream) {
     const void* fn = p.N == 16 ? stream_fn_16() : p.N == 32 ? stream_fn_32() : stream_fn_64();
     static bool attr[kDeviceSlots][3] = {};
-    const int dev = device_slot();
+    const int dev = p.dev;
     if (dev < 0) return cudaErrorInvalidDevice;
     const int idx = p.N == 16 ? 0 : p.N == 32 ? 1 : 2;
     if (!attr[dev][idx]) {
@@ -72,7 +71,7 @@ cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32
 }
 
 cudaError_t launch_warpseg(const Params& p, int64_t grid, cudaStream_t stream, bool early) {
-    if (warpseg_ctas_per_sm(p.N, p.algo) < 1) return cudaErrorInvalidConfiguration;
+    if (warpseg_ctas_per_sm(p.N, p.algo, p.dev) < 1) return cudaErrorInvalidConfiguration;
     if (grid < 1) return cudaSuccess;
     return launch_params(ws_fn(p.N, p.algo == 2), grid, kWsThreads, ws_smem(p.N), p, stream,
                          early);

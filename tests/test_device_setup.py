@@ -63,7 +63,7 @@ const void* stream_fn_64() { return &k[8]; }
 cudaError_t launch_warpseg(const Params& p, int64_t grid, cudaStream_t stream, bool early);
 cudaError_t launch_stream(const Params& p, int64_t chunk, int64_t seg_len, int32_t maxseg,
                           int32_t foreign, cudaStream_t stream);
-int warpseg_ctas_per_sm(int N, int algo);
+int warpseg_ctas_per_sm(int N, int algo, int dev);
 }
 
 int main() {
@@ -73,9 +73,10 @@ int main() {
                 sosf::Params p{};
                 p.N = N;
                 p.C = 1;
+                p.dev = sosf::device_slot();
                 for (int algo = 1; algo <= 2; ++algo) {
                     p.algo = algo;
-                    if (sosf::warpseg_ctas_per_sm(N, algo) != 2 + g_dev) ++g_failed;
+                    if (sosf::warpseg_ctas_per_sm(N, algo, g_dev) != 2 + g_dev) ++g_failed;
                     if (sosf::launch_warpseg(p, 4, nullptr, true) != cudaSuccess) ++g_failed;
                 }
                 if (sosf::launch_stream(p, 100, 100, 1, 0, nullptr) != cudaSuccess) ++g_failed;
