@@ -103,8 +103,8 @@ typedef enum sos_status {
  *             bit 4 (SOS_FLAG_DOUBLE_FLOAT): run every channel within its
  *             memory horizon with double-float samples (precision class 3
  *             of sos_plan_extended), whatever the plan's estimate; about five
- *             times the arithmetic, for results within about 2^-40 of the
- *             exact ones where FP32 would lose digits.
+ *             times the arithmetic, for results rounded to FP32 once: the
+ *             samples handed from section to section carry about 40 bits.
  *             bits 8..11 (SOS_FLAG_WS_CTAS(n)): CTAs per SM of the
  *             warp-segment launch, 1..15 (0 = as many as fit; more than fit
  *             is clamped).  Fewer, longer-running warps suit calls whose
@@ -435,7 +435,8 @@ sos_status sos_plan_query(void *workspace, int32_t first, int32_t count, int32_t
  *      basis in which those powers are small (s1 = z1, s2 = (z2 - a1 z1 / 2) /
  *      w), and channels with P > 8192 run the scan and fold (S4) in
  *      double-float;
- *   3  sections run with double-float samples (about 44 bits): the plan's
+ *   3  sections run with double-float samples (about 40 bits; on channels with
+ *      P > 8192 about 44): the plan's
  *      estimate of the error that FP32 rounding of the signal handed from
  *      section k to k + 1 would cause at the output (white input, from the
  *      norms of the partial cascades by partial fractions) exceeds 2^-15 for

@@ -1201,8 +1201,7 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         out32->ab = make_float4((float)a1, (float)a2, (float)(b1 * sb), (float)(b2 * sb));
         out32->alo = make_float4((float)(a1 - (double)(float)a1), (float)(a2 - (double)(float)a2),
                                  0.0f, 0.0f);
-        const bool twice = m > kRefineEntry || sens > kRefineSens;
-        out32->misc = make_float4((float)b0, (float)s_G[k], s_Ginv[k], twice ? 3.f : ext);
+        out32->misc = make_float4((float)b0, (float)s_G[k], s_Ginv[k], ext);
         out32->braw = make_float4((float)b0, (float)b1, (float)b2, 0.0f);
         out32->blo = make_float4((float)(b0 - (double)(float)b0), (float)(b1 - (double)(float)b1),
                                  (float)(b2 - (double)(float)b2), 0.0f);

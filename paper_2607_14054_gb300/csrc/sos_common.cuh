@@ -185,16 +185,17 @@ struct __align__(16) Coef32 {
 // coefficients' low parts (two FMAs per sample and pass): the output's
 // relative error from rounding a1, a2 is about the displacement.  The states
 // are scanned in a basis in which no power's entry is large, so the scan needs
-// no more than FP32.  misc.w is 3 for the few sections of level 2 whose FP32
-// solve may be off by more than about 1e-4 (poles within about 1/64 of z = +-1):
-// in a double-float range they get a second round of refinement (measured with
-// the refined solve on channels of radius 0.999..0.9999 too: one round
-// everywhere left one of 64 channels at 1.1e-2 instead of 4e-4 and changed no
-// other; two rounds at all of level 2 took 14.5 instead of 11.9 ms).
+// no more than FP32.  In a double-float range sections of both levels get a
+// second round of refinement: one leaves the error of an FP32 solve squared, 2^-40
+// for poles away from the axis but more next to it.  Low-passes at 0.003..0.05
+// twice before high-passes twice: worst of 178 channels 2.7e-6 step by step in
+// double-float, 1.4e-6 with the second round at the worst sections only, 6.2e-8
+// so; 64 channels of radius 0.999..0.9999 streamed, 1.1e-5, 7.9e-6 and 3.2e-6.
+// It costs 1 % of the crossover's call (16 channels of 100,003) and 2 % of the
+// batch of 4096; at level 0 too it would cost 40 % of a call all in double-float
+// and changed no error.
 constexpr float kDfScanEntry = 8.f;
 constexpr double kDfCoefSens = 1e-4;
-constexpr float kRefineEntry = 64.f;
-constexpr float kRefineSens = 1e-3f;
 constexpr double kAloCoefSens = 0x1p-18;
 
 // A channel is run with double-float samples throughout (ChanInfo::ext = 3)

@@ -153,8 +153,8 @@ __device__ __forceinline__ void ws_stage(const Coef32* cf0, const CoefDF* cx, in
 
 // Sections [k0, k1) of a channel run with double-float samples over one
 // group (kPrecDF): on entry the lane's row holds its chunk of the range's
-// FP32 input, on exit the chunk of its output, rounded once.  The most
-// ill-conditioned sections get a second round of refinement.
+// FP32 input, on exit the chunk of its output, rounded once.  Sections of level
+// 1 and 2 get a second round of refinement.
 template <int N, bool ZF>
 __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int owner, int mq) {
     const Params& p = s_ws.p;
@@ -179,7 +179,7 @@ __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int
         df z1{zz.x, zz.y}, z2{zz.z, zz.w};
         pipe_section_dfx<N, ZF>(xh, xl, mx, sd, sc[k].phi,
                                 make_float2(sc[k].cpl.x, sc[k].cpl.y),
-                                sc[k].misc.w > 2.5f ? 2 : 1, z1, z2, lane == owner, mq, row,
+                                sc[k].misc.w > 0.5f ? 2 : 1, z1, z2, lane == owner, mq, row,
                                 zf_dst);
         if (lane == 0) zs[k] = make_float4(z1.hi, z1.lo, z2.hi, z2.lo);
     }
