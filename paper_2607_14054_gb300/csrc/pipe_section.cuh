@@ -428,6 +428,9 @@ __device__ __forceinline__ void q_history(const QChunk<N>& v, int j, f2x& hu, f2
     hw = f2_pack(ub, wa);
 }
 
+// The largest magnitude in the lane's chunk (NaN skipped); for a chunk that holds
+// an infinite sample the largest of the other lanes', so that the samples before
+// it keep the digits that their own magnitude gives them.
 template <int N>
 __device__ __forceinline__ float q_max(const QChunk<N>& v) {
     float m = 0.f;
@@ -437,6 +440,11 @@ __device__ __forceinline__ float q_max(const QChunk<N>& v) {
         f2_unpack(v.u[i], a, b);
         f2_unpack(v.w[i], c, d);
         m = fmaxf(fmaxf(m, fmaxf(fabsf(a), fabsf(b))), fmaxf(fabsf(c), fabsf(d)));
+    }
+    if (__any_sync(0xffffffffu, m == INFINITY)) {
+        float f = m < INFINITY ? m : 0.f;
+        for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
+        if (m == INFINITY) m = f;
     }
     return m;
 }
@@ -477,7 +485,8 @@ __device__ __forceinline__ float sum_anchor(float bound) {
 template <int N, bool ZF = false>
 __device__ __forceinline__ void pipe_section_dfx(QChunk<N>& xh, QChunk<N>& xl, float& mx,
                                                  const SecDF& q, const float4* phi,
-                                                 const float2 cpl, int refine, df& Z1, df& Z2, bool zf_owner, int mq, float* row,
+                                                 const float2 cpl, int refine, df& Z1, df& Z2,
+                                                 bool zf_owner, int mq, float* row,
                                                  float* zf_dst) {
     constexpr int Q = N / 4;
     const int lane = threadIdx.x & 31;
