@@ -120,10 +120,11 @@ typedef enum sos_status {
  * tile counts sos_plan_query reports stay those of segments of at least 2 P)
  * that each start P samples early from zero state (no cross-segment
  * dependency).  Channels with P > 8192 keep segments of 2 P and have each run
- * by a team of up to four warps, one per share of the sections.  Coincident
- * poles, where partial fractions fail, get a cruder bound over the largest
- * pole radius r (a tail of the form C(n + 2K - 1, 2K - 1) r^n) when the
- * channel is at least eight of the segments it asks for.  Where no horizon is
+ * by a team of up to four warps, one per share of the sections (with PH).
+ * Coincident poles, where partial fractions fail, get a cruder bound over the
+ * largest pole radius r (a tail of the form C(n + m - 1, m - 1) r^n, of whose
+ * energy 2^-22 is dropped) when the channel is at least eight of the segments
+ * it asks for.  Where no horizon is
  * bounded (a pole within 1e-7 of the unit circle, or coincident poles on a
  * shorter channel), the DF2T state of every section is carried by a
  * decoupled look-back composing FP64-accurate affine maps (Sec. V's group
@@ -434,9 +435,9 @@ sos_status sos_plan_query(void *workspace, int32_t first, int32_t count, int32_t
  *      N = 64) or a displacement beyond 1e-4: its scan state is kept in a
  *      basis in which those powers are small (s1 = z1, s2 = (z2 - a1 z1 / 2) /
  *      w), and channels with P > 8192 run the scan and fold (S4) in
- *      double-float;
- *   3  sections run with double-float samples (about 40 bits; on channels with
- *      P > 8192 about 44): the plan's
+ *      double-float (sos_filter, sos_apply and sos_filtfilt with PH);
+ *   3  sections run with double-float samples (about 40 bits; about 44 where
+ *      class 2 has its double-float scan): the plan's
  *      estimate of the error that FP32 rounding of the signal handed from
  *      section k to k + 1 would cause at the output (white input, from the
  *      norms of the partial cascades by partial fractions) exceeds 2^-15 for

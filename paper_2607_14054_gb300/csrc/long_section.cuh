@@ -1,12 +1,15 @@
-// Sections of long-memory channels (horizon above kLongHorizon): one scalar
-// chain per lane, ill-conditioned sections with the lane scan in double-float,
-// and sections with double-float samples step by step.  The rounding errors of
-// poles this close to the unit circle add up over 1e4 and more samples to
-// 1e-5..1e-3 of a channel's output, so that any other order of operations, as
-// good as this one against the exact result, gives visibly other digits; such
-// channels keep this order whatever the call around them.  The latency of the
-// dependent steps is what bounds a segment; a team of warps takes its sections
-// as stages of a pipeline (long_segment in warpseg.cuh).
+// Sections of long-memory channels (horizon above kLongHorizon) in sos_filter,
+// sos_apply and sos_filtfilt with PH: one scalar chain per lane, ill-conditioned
+// sections with the lane scan in double-float, and sections with double-float
+// samples step by step.  The rounding errors of poles this close to the unit
+// circle add up over 1e4 and more samples to 1e-5..1e-3 of a channel's output, in
+// any order of operations, but other ones in each: this one is kept for its
+// digits.  (Streams and plans for cyclic reduction run the same channels by
+// pipe_section and pipe_section_dfx, whose errors are no larger: 64 channels of 8
+// sections, radius 0.999..0.9999, by class: level 2 at most 1.6e-3 here and 4.4e-4
+// there, class 3 4.9e-4 and 2.1e-4.)  The latency of the dependent steps is what
+// bounds a segment; a team of warps takes its sections as stages of a pipeline
+// (ws_long_phase in warpseg.cuh).
 #pragma once
 
 #include "pipe_section.cuh"
