@@ -1355,8 +1355,9 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
     // ---- prefixes: look-back tiles of the carried channels (tb, by
     // channel) and segments of the channels within their horizon (tbp, by
     // dispatch position: porder lists the long-memory channels first, and
-    // before the others of each kind the channels of precision class 3, their segments costing several times the others', so that they
-    // are handed out first and do not trail the launch) ----
+    // before the others of each kind the channels of precision class 3, their
+    // segments costing several times the others', so that they are handed out
+    // first and do not trail the launch) ----
     __shared__ int64_t s_carry2;
     __shared__ int64_t s_wsum2[32];
     // block-wide exclusive scan of one value per thread (every thread
@@ -1383,7 +1384,16 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
     }
     __syncthreads();
     int carried = 0, widest = 0;
-    // tiles of carried channels; the most sections of a long-memory channel
+    // dispatch categories: long-memory channels (double-float ones first), then
+    // the others (the same)
+    auto category = [&](int c) {
+        const bool far = __ldcg(&p.chan[c].longm) != 0;
+        const bool df3 = __ldcg(&p.chan[c].horizon) >= 0 && __ldcg(&p.chan[c].ext) >= 3;
+        return (far ? 0 : 2) + (df3 ? 0 : 1);
+    };
+    // tiles of carried channels; the most sections of a long-memory channel; the
+    // channels of each category
+    int cnt[4] = {0, 0, 0, 0};
     for (int base = 0; base < C; base += blockDim.x) {
         const int c = base + tid;
         int64_t nt = 0;
@@ -1397,35 +1407,55 @@ __device__ __noinline__ void order_pass(const Params& p, unsigned long long* s_k
                 const int K = __ldcg(&p.chan[c].K);
                 widest = widest > K ? widest : K;
             }
+            const int cat = category(c);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cnt[q] += cat == q;
         }
         const int64_t t0 = scan(nt, s_wsum, &s_carry);
         if (c < C) p.tb[c] = t0;
     }
     const int64_t total = s_carry;
     const int team = __syncthreads_or(widest > 4) ? 4 : __syncthreads_or(widest > 2) ? 2 : 1;
-    // dispatch positions: long-memory channels (double-float ones first), then
-    // the others (the same), as categories 0..3
+    // dispatch positions, all categories in one scan of four 16-bit counts (a
+    // scan for each of them: a full plan of 65,536 channels 5.65 ms instead of 5.20)
+    __shared__ int s_count[4];
+    __shared__ int64_t s_pos[4];
+    if (tid < 4) s_count[tid] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int n = __reduce_add_sync(0xffffffffu, cnt[q]);
+        if (lane == 0 && n) atomicAdd(&s_count[q], n);
+    }
+    __syncthreads();
     int64_t first_of[4];
-    for (int cat = 0; cat < 4; ++cat) {
-        first_of[cat] = s_carry2;
-        __syncthreads();
-        for (int base = 0; base < C; base += blockDim.x) {
-            const int c = base + tid;
-            int64_t f = 0;
-            if (c < C) {
-                const bool far = __ldcg(&p.chan[c].longm) != 0;
-                const bool df3 =
-                    __ldcg(&p.chan[c].horizon) >= 0 && __ldcg(&p.chan[c].ext) >= 3;
-                f = (far ? 0 : 2) + (df3 ? 0 : 1) == cat ? 1 : 0;
-            }
-            const int64_t q = scan(f, s_wsum2, &s_carry2);
-            if (c < C && f) p.porder[q] = c;
+    first_of[0] = 0;
+#pragma unroll
+    for (int q = 1; q < 4; ++q) first_of[q] = first_of[q - 1] + s_count[q - 1];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (tid == q) s_pos[q] = first_of[q];
+    for (int base = 0; base < C; base += blockDim.x) {
+        const int c = base + tid;
+        const int sh = c < C ? 16 * category(c) : 0;
+        const unsigned long long v = c < C ? 1ull << sh : 0ull;
+        unsigned long long inc = v;
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long o = __shfl_up_sync(0xffffffffu, inc, d);
+            if (lane >= d) inc += o;
         }
+        if (lane == 31) s_wsum2[warp] = (int64_t)inc;
         __syncthreads();
+        unsigned long long pre = 0, all = 0;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+            if (w == warp) pre = all;
+            all += (unsigned long long)s_wsum2[w];
+        }
+        if (c < C) p.porder[s_pos[sh >> 4] + (int64_t)(((pre + inc - v) >> sh) & 0xffff)] = c;
+        __syncthreads();
+        if (tid < 4) s_pos[tid] += (int64_t)((all >> (16 * tid)) & 0xffff);
     }
     __syncthreads();  // porder complete (block-wide visibility of its global writes)
-    if (tid == 0) s_carry2 = 0;
-    __syncthreads();
     for (int base = 0; base < C; base += blockDim.x) {
         const int i = base + tid;
         int64_t ns = 0;
