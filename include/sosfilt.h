@@ -67,8 +67,8 @@ typedef enum sos_status {
 
 /* Tuning knobs.  Pass NULL for the library defaults.
  *   n_blocks: N, samples per lane per group (the paper's number of blocks):
- *             16, 32 or 64 (0 = default: 64, or 32 where warps is given; 32
- *             for the backward).
+ *             16, 32 or 64 (0 = default: 64, or 32 where warps or
+ *             SOS_FLAG_SECTION_PIPELINE is given; 32 for the backward).
  *   warps:    W, warps per tile (one tile = W*32*N samples): 4, 8 or 16 (4
  *             not with N = 16, 16 not with N = 64; 0 = default: 4 with the
  *             default N, else 8; the backward 8).

@@ -34,11 +34,14 @@ struct Tune {
 
 // The library's defaults: N = 64, W = 4 (tiles of 8,192 samples).  N given alone
 // takes W = 8, W given alone N = 32, for which every documented W is compiled.
+// The section pipeline's default is N = 32, W = 8: its warps run one section
+// each, and a group of 2,048 samples fills and drains the pipeline slower than it
+// saves scans (2^24 samples, K = 8: 82 us, 92 at N = 64; K = 2: 48 and 60).
 bool resolve_tuning(const sos_tuning* t, Tune* out) {
     Tune r{64, 4, 1, 0, 0, 0};
     bool chosen = false;
     if (t) {
-        if (t->n_blocks || t->warps) {
+        if (t->n_blocks || t->warps || (t->flags & SOS_FLAG_SECTION_PIPELINE)) {
             r.N = t->n_blocks ? t->n_blocks : 32;
             r.W = t->warps ? t->warps : 8;
             chosen = true;

@@ -47,6 +47,15 @@ def test_default_carries_with_n32(kmax):
     assert torch.equal(_channels(plan(x, sos, K, zi)[0], lengths)[4], y64[4])
 
 
+def test_section_pipeline_default():
+    """The section pipeline's flag alone takes N = 32 and W = 8."""
+    P = _lib()
+    lengths = [9000, 70_001, 1, 20_011]
+    x, sos, K, L, zi = (a.cuda() for a in random_case(735, lengths, 6, rmax=0.97))
+    out = [P.SosFilter(lengths, 6, tuning=t)(x, sos, K, zi) for t in ((0, 0, 0, 4), (32, 8, 1, 4))]
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
 def test_carried_beside_segments():
     """Coincident poles on a short channel (carried) and others in one call."""
     P = _lib()
