@@ -13,7 +13,8 @@ look-back (poles near the unit circle): only then does W, the look-back
 kernel's tile width, matter, so only then are several W tried.  And whether
 some section is ill-conditioned for FP32 (``SosFilter.plan_extended``): only
 the PH warp-segment kernel gives those sections extended precision, so then
-neither the section pipeline nor cyclic reduction is a candidate, nor N = 64.
+neither the section pipeline nor cyclic reduction is a candidate.  The library's
+own default is always one.
 """
 from __future__ import annotations
 
@@ -29,7 +30,7 @@ import torch
 SUPPORTED_NW = [(16, 8), (16, 16), (32, 4), (32, 7), (32, 8), (32, 16), (64, 3), (64, 4), (64, 7),
                 (64, 8)]
 ALGOS = (1, 2)  # PH, cyclic reduction
-DEFAULT = (32, 8, 1, 0)
+DEFAULT = (0, 0, 0, 0)  # the library's own choice (N = 64 segments, N = 32 look-back)
 
 _cache: Dict[Tuple, Tuple[int, int, int, int]] = {}
 _lock = threading.Lock()
@@ -59,7 +60,7 @@ def ws_ctas(n: int) -> int:
 # calls whose segments fill the GPU about once), and the section pipeline
 KERNELS = {16: (0, ws_ctas(2), SECTION_PIPELINE),
            32: (0, ws_ctas(2), SECTION_PIPELINE),
-           64: (0, ws_ctas(2), SECTION_PIPELINE)}
+           64: (0, SECTION_PIPELINE)}  # two CTAs per SM are what fits
 
 
 def candidates(carried: bool, extended: bool = False) -> List[Tuple[int, int, int, int]]:
@@ -69,8 +70,8 @@ def candidates(carried: bool, extended: bool = False) -> List[Tuple[int, int, in
     the warp-segment kernel with N <= 32 only when some section is
     ill-conditioned."""
     out = []
-    # ill-conditioned sections: N <= 32 (the in-lane FP32 runs are N samples
-    # long; at N = 64 some precision-stress channels exceed the FP32 bound)
+    # ill-conditioned sections: N <= 32, whose in-lane FP32 runs are shorter (at
+    # N = 64 the default, which autotune() adds, stands for the others)
     for n in ((16, 32) if extended else (16, 32, 64)):
         ws = sorted({w for (nn, w) in SUPPORTED_NW if nn == n}) if carried else \
             [8 if (n, 8) in SUPPORTED_NW else min(w for (nn, w) in SUPPORTED_NW if nn == n)]
@@ -131,7 +132,8 @@ def _time_apply(plan, x, y, zi, zf, sos, K, reps: int) -> float:
 def autotune(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] = None,
              lengths=None, zi: Optional[torch.Tensor] = None, reps: int = 5,
              use_cache: bool = True, report: Optional[list] = None) -> Tuple[int, int, int, int]:
-    """Fastest (N, W, algo, flags) for this call's shapes, by measurement."""
+    """Fastest (N, W, algo, flags) for this call's shapes, by measurement (zeros:
+    the library's default)."""
     from . import SosFilter
     sos = sos if sos.dim() == 3 else sos.unsqueeze(0)
     C, kmax = int(sos.shape[0]), int(sos.shape[1])
@@ -156,7 +158,7 @@ def autotune(x: torch.Tensor, sos: torch.Tensor, K: Optional[torch.Tensor] = Non
     y = torch.empty_like(x)
     zf = torch.empty((C, kmax, 2), dtype=torch.float32, device=x.device)
     best, best_t = DEFAULT, float("inf")
-    for cand in candidates(carried, extended):
+    for cand in [DEFAULT] + candidates(carried, extended):
         plan = SosFilter(lh, kmax, tuning=cand, device=x.device)
         t = _time_apply(plan, x, y, zi, zf, sos.contiguous(), K, reps)
         if report is not None:
