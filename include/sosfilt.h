@@ -123,7 +123,7 @@ typedef enum sos_status {
  * by a team of up to four warps, one per share of the sections (with PH).
  * Coincident poles, where partial fractions fail, get a cruder bound over the
  * largest pole radius r (a tail of the form C(n + m - 1, m - 1) r^n, of whose
- * energy 2^-22 is dropped) when the channel is at least eight of the segments
+ * energy at most 2^-21 is dropped) when the channel is at least eight of the segments
  * it asks for.  Where no horizon is
  * bounded (a pole within 1e-7 of the unit circle, or coincident poles on a
  * shorter channel), the DF2T state of every section is carried by a

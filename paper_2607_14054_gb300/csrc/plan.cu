@@ -597,7 +597,7 @@ __device__ float response_log_norm(const double (*rows)[5], const float (*rowsf)
 // same bound but for sections whose pole pair lies far enough from the axis for
 // r^n / sin(angle) to be less than (n + 1) r^n over P samples: their
 // coefficients are then those of one factor, not two.  For two equal sections it
-// comes to P again (4,464 for 4,416 samples at a cutoff of 0.002).
+// comes to P again (4,416 samples at a cutoff of 0.002).
 // One warp, the same result in every lane.
 __device__ int horizon_fallback(const double (*rows)[5], const float (*rowsf)[5], int K, float h2,
                                 int lane, int& tz, int& warm) {

@@ -108,9 +108,12 @@ static_assert(sizeof(ChanInfo) == 80, "channel table entry");
 // unit circle, coincident poles) keep the decoupled look-back.
 constexpr float kHorizonEps = 0x1p-30f;
 // Coincident poles' warm-up (horizon_fallback): the energy of the response's
-// dropped tail relative to ||h||_2.  What a segment drops it drops over its first
-// 1 / (1 - r) samples, a few per cent of it: below FP32's rounding of the output.
-constexpr float kFallbackEps = 0x1p-22f;
+// dropped tail relative to ||h||_2, by a bound that is itself 2 to 8 times the
+// tail.  What a segment drops it drops over its first 1 / (1 - r) samples, a few
+// per cent of it: about FP32's rounding of the output.  (At 2^-22 two equal
+// sections would be warmed up over 1 % more than before, which for a small call
+// may be a group more in three.)
+constexpr float kFallbackEps = 0x1p-21f;
 
 // Channels with a longer horizon keep the scalar order of operations of
 // long_section.cuh on the warp-segment kernel (there the reason), in segments

@@ -2,10 +2,11 @@
 partial fractions, in double-float against the FP64 oracle: what their segments
 drop stays below FP32's rounding.
 
-Tolerance.  The tail that a segment drops has an energy of at most 2^-22 =
-2.4e-7 of the response's, so 2.4e-7 of a white input's output at the segment's
-first samples and less after them; the output is rounded once (6e-8) and the
-sections' double-float adds less: 5e-7 relative L2."""
+Tolerance.  The tail that a segment drops has an energy of at most 2^-21 =
+4.8e-7 of the response's, so 4.8e-7 of a white input's output at the segment's
+first samples, and less than half of that over the whole segment, which is
+several of the response's decay times long; the output is rounded once (6e-8)
+and the sections' double-float adds less: 5e-7 relative L2."""
 import math
 
 import numpy as np

@@ -2,7 +2,7 @@
 CPU against FP64 impulse responses: with r the largest pole radius, A = prod_k
 B_k r^-2 (B_k = |b0| + |b1| + |b2|) and the pole pairs far from the axis counted
 as one factor of 1 / sin(angle) r^n instead of two, the tail's energy from the
-first n on where A' C(n + m - 1, m - 1) r^n / sqrt(1 - ratio^2) is below 2^-22
+first n on where A' C(n + m - 1, m - 1) r^n / sqrt(1 - ratio^2) is below 2^-21
 ||h||_2 is below that too; and the norm of 32 points across the nearest poles'
 peaks is one from below."""
 import math
@@ -44,7 +44,7 @@ def _warm_up(rows, P, norm):
     with np.errstate(invalid="ignore", divide="ignore"):
         t = (loga + n * math.log(r) + sum(np.log(n + i) for i in range(1, m))
              - 0.5 * np.log(1 - ratio ** 2))
-    ok = (ratio < 1) & (t <= math.log(2.0 ** -22 * norm))
+    ok = (ratio < 1) & (t <= math.log(2.0 ** -21 * norm))
     return int(n[np.argmax(ok)])
 
 
@@ -84,4 +84,4 @@ def test_tail_below_the_bound(idx):
     # at P = 0 every section counts twice; with P large, all complex pairs once
     for P in (0, 200, 1 << 30):
         n = _warm_up(_rows(sos), P, max(low, 1e-3 * norm))
-        assert n > 1 and np.sqrt((h[n:] ** 2).sum()) <= 2.0 ** -22 * norm, (P, n)
+        assert n > 1 and np.sqrt((h[n:] ** 2).sum()) <= 2.0 ** -21 * norm, (P, n)
