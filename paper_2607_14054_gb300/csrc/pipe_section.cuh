@@ -373,6 +373,7 @@ __device__ __forceinline__ void lane_section(float (&v)[N], const float4 ab, con
 // precision throughout (normalised by a0, never factored).
 struct SecDF {
     df a1, a2, b0, b1, b2;
+    int rounds;  // of refinement (pipe_section_dfx)
 };
 
 __device__ __forceinline__ f2x f2_neg1() { return f2_dup(-1.f); }
@@ -428,9 +429,7 @@ __device__ __forceinline__ void q_history(const QChunk<N>& v, int j, f2x& hu, f2
     hw = f2_pack(ub, wa);
 }
 
-// The largest magnitude in the lane's chunk (NaN skipped); for a chunk that holds
-// an infinite sample the largest of the other lanes', so that the samples before
-// it keep the digits that their own magnitude gives them.
+// The largest magnitude in the lane's chunk (NaN skipped).
 template <int N>
 __device__ __forceinline__ float q_max(const QChunk<N>& v) {
     float m = 0.f;
@@ -441,12 +440,16 @@ __device__ __forceinline__ float q_max(const QChunk<N>& v) {
         f2_unpack(v.w[i], c, d);
         m = fmaxf(fmaxf(m, fmaxf(fabsf(a), fabsf(b))), fmaxf(fabsf(c), fabsf(d)));
     }
-    if (__any_sync(0xffffffffu, m == INFINITY)) {
-        float f = m < INFINITY ? m : 0.f;
-        for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
-        if (m == INFINITY) m = f;
-    }
     return m;
+}
+
+// q_max of a group with infinite samples: a lane that has one takes the largest
+// of the others, so that the samples before it keep the digits that their own
+// magnitude gives them.
+__device__ __forceinline__ float finite_max(float m) {
+    float f = m < INFINITY ? m : 0.f;
+    for (int o = 16; o > 0; o >>= 1) f = fmaxf(f, __shfl_xor_sync(0xffffffffu, f, o));
+    return m < INFINITY ? m : f;
 }
 
 // 1.5 * 2^e such that sums of terms up to `bound` in absolute value, added to
@@ -478,13 +481,13 @@ __device__ __forceinline__ float sum_anchor(float bound) {
 // the sum (sum_anchor): each addition's error comes back exactly from two
 // more FMAs, and the errors are summed beside the low parts.
 // xh, xl: the section's input, replaced by its output.  mx: max |x| of the
-// lane, replaced by max |y|.  Z1, Z2: the group's incoming DF2T state in
+// lane, replaced by max |y|; wild: the group's input has infinite samples.  Z1, Z2: the group's incoming DF2T state in
 // double-float, left outgoing.  refine: rounds of refinement.  ZF: the group
 // holds the channel's last sample (element mq of the chunk of the lane where
 // zf_owner is set), whose state goes to zf_dst; row: scratch for it.
 template <int N, bool ZF = false>
 __device__ __forceinline__ void pipe_section_dfx(QChunk<N>& xh, QChunk<N>& xl, float& mx,
-                                                 const SecDF& q, const float4* phi,
+                                                 bool wild, const SecDF& q, const float4* phi,
                                                  const float2 cpl, int refine, df& Z1, df& Z2,
                                                  bool zf_owner, int mq, float* row,
                                                  float* zf_dst) {
@@ -564,6 +567,7 @@ __device__ __forceinline__ void pipe_section_dfx(QChunk<N>& xh, QChunk<N>& xl, f
     QChunk<N> y, d;
     pole_solve<N>(xh, y, na1, na2, nl1, nl2, phi, cpl);
     mx = q_max<N>(y);
+    if (wild) mx = finite_max(mx);
 #pragma unroll 1
     for (int it = 0;; ++it) {
         const float my = fmaxf(mx, __shfl_up_sync(0xffffffffu, mx, 1));
@@ -596,6 +600,7 @@ __device__ __forceinline__ void pipe_section_dfx(QChunk<N>& xh, QChunk<N>& xl, f
             y.w[m] = f2_add(y.w[m], d.w[m]);
         }
         mx = q_max<N>(y);
+        if (wild) mx = finite_max(mx);
     }
     // y + d as hi and lo parts
 #pragma unroll

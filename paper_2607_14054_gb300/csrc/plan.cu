@@ -96,6 +96,15 @@ __device__ __forceinline__ float coef_sensitivity(double a1, double a2) {
     return (r * da1 + da2) / (sep * gap);
 }
 
+// ||g||^2, g the impulse response of 1 / (1 + a1 z^-1 + a2 z^-2): what white noise
+// put into the recursion comes out with.  Infinite for a pole on or outside the
+// unit circle.
+__device__ __forceinline__ double pole_gain2(double a1, double a2) {
+    const double d = (1.0 - a2) * ((1.0 + a2) * (1.0 + a2) - a1 * a1);
+    if (!(d > 0.0) || !(1.0 + a2 > 0.0)) return INFINITY;
+    return (1.0 + a2) / d;
+}
+
 // Condition number of one normalised section, kappa = ||g|| ||b|| / ||h||:
 // g the impulse response of 1 / (1 + a1 z^-1 + a2 z^-2), h that of the whole
 // section, b = (b0, b1, b2).  Closed forms from the autocorrelation of the
@@ -105,9 +114,8 @@ __device__ __forceinline__ float coef_sensitivity(double a1, double a2) {
 // outside the unit circle or a vanishing response.  FP64, one lane.
 __device__ __forceinline__ double section_kappa(double b0, double b1, double b2, double a1,
                                                 double a2) {
-    const double d = (1.0 - a2) * ((1.0 + a2) * (1.0 + a2) - a1 * a1);
-    if (!(d > 0.0) || !(1.0 + a2 > 0.0)) return INFINITY;
-    const double c0 = (1.0 + a2) / d;
+    const double c0 = pole_gain2(a1, a2);
+    if (!isfinite(c0)) return INFINITY;
     const double c1 = -a1 * c0 / (1.0 + a2);
     const double c2 = -a1 * c1 - a2 * c0;
     const double bb = b0 * b0 + b1 * b1 + b2 * b2;
@@ -1188,9 +1196,13 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
         }
         for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
+    bool hard = false;
+    float gain2 = 0.f;
     if (lane == 0) {
         // extended precision (FP64 work on one lane: the FP64 pipe is narrow)
         const float sens = coef_sensitivity(a1, a2);
+        hard = m > kRefineEntry || sens > kRefineSens;
+        gain2 = (float)pole_gain2(a1, a2);
         const float ext = (m > kDfScanEntry || sens > (float)kDfCoefSens)
                               ? 2.f
                               : (sens > (float)kAloCoefSens ? 1.f : 0.f);
@@ -1210,6 +1222,17 @@ __device__ __forceinline__ bool plan_channel(const Params& p) {
     // ---- Psi = A^(NL) and Theta = A^T, only for channels carried by the
     // look-back (its warp and tile steps) ----
     asm volatile("bar.sync 2, %0;" ::"r"(32 * (Kc + 2)) : "memory");
+    if (lane == 0) {
+        // rounds of refinement in a double-float range (sos_common.cuh)
+        float amp = s_handoff * 0x1p24f;
+        if (!(amp >= 0.f)) {
+            bool equal = true;
+            for (int j = 1; j < Kc; ++j)
+                for (int i = 0; i < 5; ++i) equal = equal && s_row[j][i] == s_row[0][i];
+            amp = equal ? 1.f : kRefineUnknown;
+        }
+        out32->braw.w = hard || gain2 * amp > kRefineGain ? 2.f : 1.f;
+    }
     if (k == 0 && lane == 0) {
         // the channel's precision class: the largest section level, or 3
         // (double-float samples) for a channel within its memory horizon

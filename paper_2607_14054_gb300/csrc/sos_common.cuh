@@ -145,7 +145,8 @@ __host__ __device__ constexpr int ext_n(int N) { return N == 64 ? 32 : N; }
 struct __align__(16) Coef32 {
     float4 ab;            // a1, a2, b1, b2  (b1, b2 divided by b0 when factored)
     float4 misc;          // b0, G_k (cumulative gain), 1/G_k, precision level
-    float4 braw;          // b0, b1, b2 normalised by a0 only (the adjoint's FIR)
+    float4 braw;          // b0, b1, b2 normalised by a0 only (the adjoint's FIR); rounds of
+                          // refinement in a double-float range
     // read together by the warp-segment kernel and the section pipeline: the
     // powers Phi^(2^j), j = 0..4 (lane scan), A^(N/2) and A^(N/4) (the joins of a
     // lane chunk's quarters) in the basis s1 = z1, s2 = (z2 - (a1/2) z1) / w, and w,
@@ -188,18 +189,29 @@ struct __align__(16) Coef32 {
 // coefficients' low parts (two FMAs per sample and pass): the output's
 // relative error from rounding a1, a2 is about the displacement.  The states
 // are scanned in a basis in which no power's entry is large, so the scan needs
-// no more than FP32.  In a double-float range sections of both levels get a
-// second round of refinement: one leaves the error of an FP32 solve squared, 2^-40
-// for poles away from the axis but more next to it.  Low-passes at 0.003..0.05
-// twice before high-passes twice: worst of 178 channels 2.7e-6 step by step in
-// double-float, 1.4e-6 with the second round at the worst sections only, 6.2e-8
-// so; 64 channels of radius 0.999..0.9999 streamed, 1.1e-5, 7.9e-6 and 3.2e-6.
-// It costs 1 % of the crossover's call (16 channels of 100,003) and 2 % of the
-// batch of 4096; at level 0 too it would cost 40 % of a call all in double-float
-// and changed no error.
+// no more than FP32.
 constexpr float kDfScanEntry = 8.f;
 constexpr double kDfCoefSens = 1e-4;
 constexpr double kAloCoefSens = 0x1p-18;
+
+// Rounds of refinement of a section in a double-float range (pipe_section_dfx;
+// Coef32::braw.w).  An FP32 solve is off by about e = 2^-23 ||g|| relative (its
+// roundings, passed by the all-pole part's response g) and one round leaves e^2,
+// which what follows the section passes on amplified by up to `amp` (2^24 times
+// handoff_error): a second round where e^2 amp > 2^-24, that is ||g||^2 amp >
+// 2^22.  amp is 1 for equal sections, whose peaks coincide, and taken as 2^16
+// where it is not known otherwise, so that e^2 stays below 2^-40 there; sections
+// within 1/64 of z = +-1 or whose poles FP32 coefficients displace by more than
+// 1e-3 of their distance to the circle always get two.  A low-pass at 0.005
+// twice before a high-pass at 0.4 twice: 1.5e-5 with the last rule alone, 2.5e-7
+// so; 178 such cascades 1.4e-6 and 6.2e-8 (2.7e-6 step by step in double-float).
+// Two rounds wherever a section is flagged made the calls of crossovers at
+// 0.0025..0.005 a third slower (72 -> 97 us for 24 channels of 94,516) and
+// changed none of their errors, which their output's rounding bounds (2.7e-8).
+constexpr float kRefineGain = 0x1p22f;
+constexpr float kRefineUnknown = 0x1p16f;
+constexpr float kRefineEntry = 64.f;
+constexpr float kRefineSens = 1e-3f;
 
 // A channel is run with double-float samples throughout (ChanInfo::ext = 3)
 // when the relative error that FP32 rounding of the signals handed from one

@@ -134,7 +134,7 @@ enum WsPrec {
 __device__ __forceinline__ SecDF load_secdf(const Coef32* cf) {
     const float4 ab = cf->ab, alo = cf->alo, br = cf->braw, bl = cf->blo;
     return SecDF{df{ab.x, alo.x}, df{ab.y, alo.y}, df{br.x, bl.x}, df{br.y, bl.y},
-                 df{br.z, bl.z}};
+                 df{br.z, bl.z}, br.w > 1.5f ? 2 : 1};
 }
 
 // the copies of a channel's K sections, one cp.async group; cx: where the
@@ -153,8 +153,7 @@ __device__ __forceinline__ void ws_stage(const Coef32* cf0, const CoefDF* cx, in
 
 // Sections [k0, k1) of a channel run with double-float samples over one
 // group (kPrecDF): on entry the lane's row holds its chunk of the range's
-// FP32 input, on exit the chunk of its output, rounded once.  Sections of level
-// 1 and 2 get a second round of refinement.
+// FP32 input, on exit the chunk of its output, rounded once.
 template <int N, bool ZF>
 __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int owner, int mq) {
     const Params& p = s_ws.p;
@@ -171,15 +170,17 @@ __device__ __forceinline__ void dfx_group(int k0, int k1, int c, int row_at, int
         xl.w[m] = 0;
     }
     float mx = q_max<N>(xh);
+    const bool wild = __any_sync(0xffffffffu, mx == INFINITY);
+    if (wild) mx = finite_max(mx);
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
         const SecDF sd = load_secdf(cf0 + k);
         float* zf_dst = ZF ? p.zf + ((int64_t)c * p.kmax + k) * 2 : nullptr;
         const float4 zz = zs[k];
         df z1{zz.x, zz.y}, z2{zz.z, zz.w};
-        pipe_section_dfx<N, ZF>(xh, xl, mx, sd, sc[k].phi,
+        pipe_section_dfx<N, ZF>(xh, xl, mx, wild, sd, sc[k].phi,
                                 make_float2(sc[k].cpl.x, sc[k].cpl.y),
-                                sc[k].misc.w > 0.5f ? 2 : 1, z1, z2, lane == owner, mq, row,
+                                sd.rounds, z1, z2, lane == owner, mq, row,
                                 zf_dst);
         if (lane == 0) zs[k] = make_float4(z1.hi, z1.lo, z2.hi, z2.lo);
     }
