@@ -88,12 +88,6 @@ int device_sms(int dev) {
 
 constexpr int kPipeCtasPerSm = 2;
 
-// Tile length: long enough that the warm-up before each tile is a small
-// fraction of it, short enough that the tiles of the whole call keep every
-// consumer busy: each pipeline CTA (between 8 and 64 groups of 32 N), or, for
-// the warp-segment kernel, each of twelve warps per SM (at least 8192 samples
-// and at most 64 groups; it cuts its own segments, Params::wseg, except those
-// of long-memory channels).
 // CTAs per SM of a warp-segment launch: the tuning's request (flag bits
 // 8..11), at most as many as fit; 0 = as many as fit.
 int warpseg_ctas(int N, int algo, int flags, int dev) {
@@ -102,6 +96,12 @@ int warpseg_ctas(int N, int algo, int flags, int dev) {
     return req > 0 && req < fit ? req : fit;
 }
 
+// Tile length: long enough that the warm-up before each tile is a small
+// fraction of it, short enough that the tiles of the whole call keep every
+// consumer busy: each pipeline CTA (between 8 and 64 groups of 32 N), or, for
+// the warp-segment kernel, each of twelve warps per SM (at least 8192 samples
+// and at most 64 groups; it cuts its own segments, Params::wseg, except those
+// of long-memory channels).
 int64_t segment_length(int64_t total_len, int N, int flags, bool warp_segments, int sms) {
     const int64_t group = 32LL * N;
     int64_t units = (int64_t)sms * kPipeCtasPerSm, gmin = 8;

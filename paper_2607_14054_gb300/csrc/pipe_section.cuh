@@ -1,8 +1,10 @@
 // One section of the cascade over one group of 32 N samples held as lane
 // chunks in registers: S3 non-recursive stage, S4-PH (particular solution,
 // lane scan, re-run from the true lane state), the group's outgoing DF2T
-// state, and S8 (zf) for the lane holding the channel's last sample.  Used
-// by the forward section pipeline and, on time-reversed data, by the adjoint.
+// state, and S8 (zf) for the lane holding the channel's last sample.  Used by the
+// warp-segment and streaming kernels and the section pipeline (pipe_section,
+// pipe_section_dfx, pipe_section_cr), by the backward (lane_section) and, on
+// time-reversed data, by its adjoint (pipe_section_dual).
 #pragma once
 
 #include "sos_f2.cuh"
@@ -772,7 +774,7 @@ __device__ __forceinline__ void pipe_section_cr(float (&v)[N], const float4 ab, 
 // gets the all-pole part (lambda, from state (L1, L2)), u the whole section
 // with coefficients (b0, b1, b2) (dL/du, from state (U1, U2)).  Both share
 // the poles, hence Phi^(2^j) and Phi^lane.  Same arithmetic as two
-// pipe_section calls.
+// lane_section calls (in DF2T states).
 template <int N>
 __device__ __forceinline__ void pipe_section_dual(float (&l)[N], float (&u)[N], const float a1,
                                                   const float a2, const float b0, const float b1,

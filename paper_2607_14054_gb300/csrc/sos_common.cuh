@@ -83,7 +83,7 @@ struct ChanInfo {
                       // carry); -1: the state is carried by the look-back
     int16_t single;   // 1: the whole channel is one segment (backward plans)
     int16_t ext;      // precision class: 0 FP32; 1, 2: the largest section level
-                      // (Coef32::misc.w); 3: double-float samples throughout
+                      // (Coef32::misc.w); 3: double-float samples in sections dflo..dfhi
     int64_t seg;      // segment length of a channel with a horizon (a multiple of 16)
     int32_t nseg;     // its segments
     int32_t zdecay;   // samples after which the response of an arbitrary initial state has
@@ -213,8 +213,8 @@ constexpr float kRefineUnknown = 0x1p16f;
 constexpr float kRefineEntry = 64.f;
 constexpr float kRefineSens = 1e-3f;
 
-// A channel is run with double-float samples throughout (ChanInfo::ext = 3)
-// when the relative error that FP32 rounding of the signals handed from one
+// A channel is run with double-float samples (ChanInfo::ext = 3; a range of its
+// sections, or all) when the relative error that FP32 rounding of the signals handed from one
 // section to the next would cause at the output, estimated by the plan for a
 // white input from zero state, exceeds kHandOffErrMax (or when the estimate
 // cannot be formed and some section needs the double-float scan), or when a

@@ -70,7 +70,7 @@ __device__ __forceinline__ void ws_load(const float* src, int64_t rem, float* sl
 
 // One warp's segment, in shared memory: what the groups' loads and stores
 // need, read where they need it, so that nothing of it is live in registers
-// through the section loop (at N = 64 the chunk alone takes 64 of the 168).
+// through the section loop (at N = 64 the chunk alone takes 64 of the 255).
 struct WsSeg {
     int64_t base;   // packed index of the first computed sample (off + cstart)
     int64_t rbase;  // packed index of that sample's mirror image in the channel
@@ -93,8 +93,9 @@ __device__ __forceinline__ int ws_cap(int64_t n) {
 // and cpl, in that order), kept by each warp in shared memory for the channel
 // of its segment: read from global memory they would be evicted from the
 // little L1 that the group slots leave by the streaming stores, a round trip
-// to L2 in every section (N = 64, 12 warps per SM, compute only: 1,214 against
-// 1,098 cycles per section of a 2048-sample group, before any store).
+// to L2 in every section (N = 64, measured with 12 warps per SM, compute only:
+// 1,214 against 1,098 cycles per section of a 2048-sample group, before any
+// store; the kernel runs eight).
 struct WsCoef {
     float4 ab, misc, phi[7], cpl;
 };
